@@ -310,12 +310,9 @@ def _roofline(alg_bytes, seconds, kernel, timing, traffic=None):
 
 
 def _eig_desc() -> str:
-    """Arithmetic of the narrow eigen-step the library runs (its default, or the
-    FP32 opt-in selected by RPCA_EIG_FP32=1)."""
-    if os.environ.get("RPCA_EIG_FP32", "0") not in ("", "0"):
-        return "T x T Jacobi with FP32 rotations and basis (opt-in); FP64 Gram sums, sigma decision, mu, test"
-    return ("T x T cyclic Jacobi in FP64 (rotations, Gram sums, basis, Newton-Schulz, Wbar; "
-            "sigma decision, mu and convergence test FP64)")
+    """Arithmetic of the narrow eigen-step."""
+    return ("FP32 one-sided Jacobi proposes the T x T eigenvectors; Gram sums, their product with it, basis and Wbar in "
+            "two-float arithmetic; sigma decision, mu and convergence test FP64")
 
 
 def _plan_pass_name(T, m, args):

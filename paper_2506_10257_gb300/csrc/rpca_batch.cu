@@ -91,7 +91,6 @@ struct rpca_batch_s {
   std::vector<PlanView> views;
   KernelInfo kern{};
   bool wide = false;           // every window runs the tiled bodies
-  int vrows = 16;              // wide eigen-steps: rows of V staged per step
   int sms = 0;
   int occ_max = 0;       // resident batch CTAs per SM the kernel allows
   BatchConfig cfg{};
@@ -308,7 +307,7 @@ void write_static_desc(rpca_batch_s* b) {
   d->nlanes = b->nlanes;
   d->paired = b->cfg.paired;
   d->spin_limit = b->spin_limit;
-  d->vrows = b->vrows;
+  d->eig_floats = (int)(b->kern.smem / sizeof(float));
   for (int l = 0; l < b->nlanes; ++l) d->lane[l] = b->lanes[l];
   for (int slot = 0; slot < b->n; ++slot) {
     const int w = b->slot_win[slot];
@@ -403,8 +402,7 @@ rpca_status rpca_batch_create(const rpca_params* params, int32_t n, rpca_batch_t
     else
       batch_tc_kernel_info(tbmax, prec == RPCA_PREC_BF16X3, &b->kern.fn, &b->kern.smem);
   } else {
-    // shared memory: the largest tiled pass or eigen-step of the batch, with
-    // as many staged V rows (<= 16) as the SM leaves room for
+    // shared memory: all that a CTA may have; every window's pass and eigen-step must fit
     const bool cplx = params[0].dtype == RPCA_C64;
     b->kern.fn = batch_wide_kernel_fn(cplx);
     cudaFuncAttributes fa;
@@ -417,20 +415,15 @@ rpca_status rpca_batch_create(const rpca_params* params, int32_t n, rpca_batch_t
     }
     const size_t room = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
     size_t need = 0;
-    for (int vr = 16; vr >= 1; --vr) {
-      need = 0;
-      for (int i = 0; i < n; ++i) {
-        const int Tr = params[i].dtype == RPCA_C64 ? 2 * params[i].T : params[i].T;
-        need = std::max({need, wide_pass_smem_bytes(wide_cw(Tr)), eig_wide_smem(Tr, vr)});
-      }
-      b->vrows = vr;
-      if (need <= room) break;
+    for (int i = 0; i < n; ++i) {
+      const int Tr = params[i].dtype == RPCA_C64 ? 2 * params[i].T : params[i].T;
+      need = std::max({need, wide_pass_smem_bytes(wide_cw(Tr)), eig_wide_smem(Tr)});
     }
     if (need > room) {
       delete b;
       return RPCA_ERR_UNSUPPORTED;
     }
-    b->kern.smem = need;
+    b->kern.smem = room / 256 * 256;  // (one CTA per SM; the eigen-steps stage their products in it)
   }
   e = cudaFuncSetAttribute(b->kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->kern.smem);
   if (e == cudaSuccess)

@@ -42,7 +42,7 @@ struct BatchDesc {
   int paired;                      // lanes of >= 2 windows and >= 3 CTAs run them two at a time (run_lane)
   unsigned long long spin_limit;   // polls of a publication wait before it gives up
   unsigned int stop;               // set once any wait ran out: every later wait gives up at once
-  int vrows;                       // wide eigen-steps: rows of V staged per step
+  int eig_floats;                  // wide eigen-steps: floats of shared memory they may use
   LaneDesc lane[kMaxLanes];
   WinDesc w[kMaxBatch];
 };
@@ -51,7 +51,7 @@ struct BatchDesc {
 __host__ __device__ constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 template <int TB>
 __host__ __device__ constexpr size_t batch_smem_tb() {
-  return cmax(pass_simt_smem<TB>(), cmax(sizeof(Eig64Smem<TB>), sizeof(EigFastSmem<TB, float>)));
+  return cmax(pass_simt_smem<TB>(), sizeof(Eig64Smem));
 }
 template <int TBMAX>
 __host__ __device__ constexpr size_t batch_smem() {
@@ -127,22 +127,13 @@ __device__ __forceinline__ void window_fail(Bufs b) {
 
 // Steps of one window kind: the narrow (register-resident) pass and eigen-step
 // for T <= kMaxT frames, or the tiled ones (wide or complex windows).
-// The eigen-step runs once per iteration and is called, not inlined, which
-// keeps the batch kernels' build short; the passes stay inlined.
-template <int TB>
-__device__ __noinline__ void narrow_eig_call(Bufs b, int flags, unsigned char* dsm) {
-  if (b.eig64)
-    eig64_body<TB>(b, flags, 0, 0, dsm);
-  else
-    eig_fast_body<TB, float>(b, flags, 0, 0, dsm);
-}
-
+// The eigen-step is called, not inlined; the passes stay inlined.
 template <int TB>
 struct NarrowBody {
   static __device__ bool pass(Bufs b, bool init, int lc, int nc, unsigned char* dsm) {
     return init ? pass_body<TB, PM_INIT>(b, lc, nc, dsm) : pass_body<TB, PM_FUSED>(b, lc, nc, dsm);
   }
-  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int) { narrow_eig_call<TB>(b, flags, dsm); }
+  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int) { eig64_body(b, flags, 0, 0, dsm); }
 };
 
 // The window's state reset before its solve (the lane's CTA 0, thread 0).
@@ -164,7 +155,7 @@ __device__ __forceinline__ void reset_window(WinDesc& wd) {
   c->rank = 0;
   c->sweeps = 0;
   c->total_sweeps = 0;
-  c->resid = 0.0;
+  c->res2 = 0.0;
   c->pass_ns = c->pass_cnt = c->eig_ns = c->eig_cnt = c->init_ns = 0ull;
   for (int i = 0; i < 4; ++i) c->eig_phase_ns[i] = 0ull;
   for (int i = 0; i < 3; ++i) c->pass_phase_ns[i] = 0ull;
@@ -223,10 +214,10 @@ __host__ __device__ inline bool lane_is_paired(int paired, const LaneDesc& ld) {
 // done flag decides it), so every wait has a matching publication; all waits
 // are bounded, and a window whose wait ran out is marked failed and its slot
 // moves on.  Disp::pass(wd, init, lc, nc, dsm) and Disp::eig(wd, flags, dsm,
-// vrows) run the window's steps for its frame bucket.
+// eig_floats) run the window's steps for its frame bucket.
 template <class Disp>
 __device__ void run_lane(BatchDesc* bd, const LaneDesc& ld, int lc, unsigned char* dsm, unsigned long long limit,
-                         unsigned int* stop, int vrows, bool paired) {
+                         unsigned int* stop, int eig_floats, bool paired) {
   const int np = paired ? ld.ncta - 1 : ld.ncta;  // pass CTAs; in a paired lane CTA np runs the eigen-steps
   const bool eigc = paired && (lc == np);
   int w[2], it[2];
@@ -247,7 +238,7 @@ __device__ void run_lane(BatchDesc* bd, const LaneDesc& ld, int lc, unsigned cha
         // ---- the eigen-step of this slot's pass it[s] ----
         if (ctr_wait(&wd.pdone, (unsigned)it[s] + 1u, limit, stop)) {
           __syncthreads();
-          Disp::eig(wd, it[s] == 0 ? (EF_INIT | EF_EIG) : (EF_CHECK | EF_EIG), dsm, vrows);
+          Disp::eig(wd, it[s] == 0 ? (EF_INIT | EF_EIG) : (EF_CHECK | EF_EIG), dsm, eig_floats);
         } else {
           window_fail(b);
         }
@@ -289,7 +280,7 @@ __device__ void run_lane(BatchDesc* bd, const LaneDesc& ld, int lc, unsigned cha
               atomicAdd(&wd.pdone, 1u);
             }
           } else {
-            Disp::eig(wd, it[s] == 0 ? (EF_INIT | EF_EIG) : (EF_CHECK | EF_EIG), dsm, vrows);
+            Disp::eig(wd, it[s] == 0 ? (EF_INIT | EF_EIG) : (EF_CHECK | EF_EIG), dsm, eig_floats);
             gen_publish(&wd.gen);
           }
         }
@@ -315,14 +306,14 @@ struct NarrowDisp {
     }
     return false;
   }
-  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int vrows) {
+  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int eig_floats) {
     switch (wd.TB) {
-      case 8: NarrowBody<8>::eig(wd.b, flags, dsm, vrows); break;
-      case 12: if constexpr (TBMAX >= 12) NarrowBody<12>::eig(wd.b, flags, dsm, vrows); break;
-      case 16: if constexpr (TBMAX >= 16) NarrowBody<16>::eig(wd.b, flags, dsm, vrows); break;
-      case 20: if constexpr (TBMAX >= 20) NarrowBody<20>::eig(wd.b, flags, dsm, vrows); break;
-      case 24: if constexpr (TBMAX >= 24) NarrowBody<24>::eig(wd.b, flags, dsm, vrows); break;
-      case 32: if constexpr (TBMAX >= 32) NarrowBody<32>::eig(wd.b, flags, dsm, vrows); break;
+      case 8: NarrowBody<8>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 12: if constexpr (TBMAX >= 12) NarrowBody<12>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 16: if constexpr (TBMAX >= 16) NarrowBody<16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 20: if constexpr (TBMAX >= 20) NarrowBody<20>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 24: if constexpr (TBMAX >= 24) NarrowBody<24>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 32: if constexpr (TBMAX >= 32) NarrowBody<32>::eig(wd.b, flags, dsm, eig_floats); break;
       default: break;
     }
   }

@@ -55,14 +55,14 @@ struct TcDisp {
     }
     return false;
   }
-  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int vrows) {
+  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int eig_floats) {
     switch (wd.TB) {
-      case 8: TcBody<8, BF16>::eig(wd.b, flags, dsm, vrows); break;
-      case 12: TcBody<12, BF16>::eig(wd.b, flags, dsm, vrows); break;
-      case 16: TcBody<16, BF16>::eig(wd.b, flags, dsm, vrows); break;
-      case 20: TcBody<20, BF16>::eig(wd.b, flags, dsm, vrows); break;
-      case 24: if constexpr (TBMAX >= 24) TcBody<24, BF16>::eig(wd.b, flags, dsm, vrows); break;
-      case 32: if constexpr (TBMAX >= 32) TcBody<32, BF16>::eig(wd.b, flags, dsm, vrows); break;
+      case 8: TcBody<8, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 12: TcBody<12, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 16: TcBody<16, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 20: TcBody<20, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 24: if constexpr (TBMAX >= 24) TcBody<24, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
+      case 32: if constexpr (TBMAX >= 32) TcBody<32, BF16>::eig(wd.b, flags, dsm, eig_floats); break;
       default: break;
     }
   }

@@ -19,8 +19,8 @@ template <int CW, int MODE, bool CPLX>
 __device__ __noinline__ bool wide_pass_call(Bufs b, int lc, int nc, float* f) {
   return pass_wide_body<CW, MODE, CPLX>(b, lc, nc, f);
 }
-__device__ __noinline__ void wide_eig_call(Bufs b, int flags, float* f, int vrows) {
-  eig_wide_body(b, flags, 0, 0, f, vrows);
+__device__ __noinline__ void wide_eig_call(Bufs b, int flags, float* f, int eig_floats) {
+  eig_wide_body<8>(b, flags, 0, 0, f, eig_floats, 0, 1);
 }
 
 template <int CW, bool CPLX>
@@ -29,8 +29,8 @@ struct WideBody {
     float* f = reinterpret_cast<float*>(dsm);
     return init ? wide_pass_call<CW, PM_INIT, CPLX>(b, lc, nc, f) : wide_pass_call<CW, PM_FUSED, CPLX>(b, lc, nc, f);
   }
-  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int vrows) {
-    wide_eig_call(b, flags, reinterpret_cast<float*>(dsm), vrows);
+  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int eig_floats) {
+    wide_eig_call(b, flags, reinterpret_cast<float*>(dsm), eig_floats);
   }
 };
 
@@ -49,8 +49,8 @@ struct WideDisp {
       default: return false;
     }
   }
-  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int vrows) {
-    wide_eig_call(wd.b, flags, reinterpret_cast<float*>(dsm), vrows);
+  static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int eig_floats) {
+    wide_eig_call(wd.b, flags, reinterpret_cast<float*>(dsm), eig_floats);
   }
 };
 
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batch_kernel_wide(BatchDesc*
   const int lc = (int)blockIdx.x - ld.cta0;
   if (lc < 0 || lc >= ld.ncta) return;
   const unsigned long long limit = bd->spin_limit;
-  const int vrows = bd->vrows;
-  run_lane<WideDisp<CPLX>>(bd, ld, lc, batch_dsm, limit, &bd->stop, vrows, lane_is_paired(bd->paired, ld));
+  const int eig_floats = bd->eig_floats;
+  run_lane<WideDisp<CPLX>>(bd, ld, lc, batch_dsm, limit, &bd->stop, eig_floats, lane_is_paired(bd->paired, ld));
 }
 
 void* batch_wide_kernel_fn(bool cplx) {

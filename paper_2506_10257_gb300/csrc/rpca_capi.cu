@@ -25,11 +25,9 @@ struct KernelSet {
   size_t pass_tc_smem[4];
   void* pass_fs[4];        // CUDA-core FP32 passes fed by TMA, by mode (needs m % 4 == 0)
   size_t pass_fs_smem;
-  void* eig64;       // plain smem Jacobi, FP64 rotations (rpca_eig on an external matrix)
-  void* eig_fast;    // the plans' eigen-step: FP64 rotations, logged and accumulated once
-  size_t eig_fast_smem;
-  void* eig_fast32;  // the same with FP32 rotations and basis arithmetic (RPCA_EIG_FP32=1)
-  size_t eig_fast32_smem;
+  void* eig64;       // FP64 Jacobi of an external matrix (rpca_eig)
+  void* eig_step;    // the plans' eigen-step
+  size_t eig_step_smem;
   int TB;
   int eig_threads;
 };
@@ -47,11 +45,9 @@ KernelSet make_set() {
   k.pass_fs[PM_UPDATE] = (void*)pass_fs_kernel<TB, PM_UPDATE>;
   k.pass_fs[PM_GRAM] = (void*)pass_fs_kernel<TB, PM_GRAM>;
   k.pass_fs_smem = FsShape<TB>::SMEM;
-  k.eig64 = (void*)eig_kernel<TB, double>;
-  k.eig_fast = (void*)eig64_kernel<TB>;
-  k.eig_fast_smem = sizeof(Eig64Smem<TB>);
-  k.eig_fast32 = (void*)eig_fast_kernel<TB, float>;
-  k.eig_fast32_smem = sizeof(EigFastSmem<TB, float>);
+  k.eig64 = (void*)eig_kernel<TB>;
+  k.eig_step = (void*)eig64_kernel;
+  k.eig_step_smem = sizeof(Eig64Smem);
   k.TB = TB;
   k.eig_threads = TB > 20 ? 512 : 256;
   return k;
@@ -102,7 +98,7 @@ bool get_set(int T, KernelSet* out) {
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t ctrl, eig, red, job, gw, ww, vw, evw, rlog, rk, rrnd, wtc, gram_part, group_part, scal_part, gscal_part, ybuf,
+  size_t ctrl, eig, red, job, gw, ww, vw, evw, escr, wtc, gram_part, group_part, scal_part, gscal_part, ybuf,
       total;
   int grid, ngroups;
   int ws_grid;     // CTAs of the passes with 128-pixel tiles (TMA-fed FP32, tiled tensor-core): one per SM
@@ -145,12 +141,7 @@ Layout make_layout(int64_t m, int T, int sms, bool wide, size_t wtc_bytes = 0) {
   L.ww = take(sizeof(float) * tw);
   L.vw = take(sizeof(float) * tw);
   L.evw = take(sizeof(double) * (size_t)T);
-  // rotation log of the wide eigen-step: every round of kWideLogSweeps sweeps
-  const size_t nrounds = wide ? (size_t)kWideLogSweeps * (size_t)(T + (T & 1)) : 1;
-  const size_t npairs = wide ? (size_t)(T + (T & 1)) / 2 : 1;
-  L.rlog = take(sizeof(float2) * nrounds * npairs);
-  L.rk = take(sizeof(int) * nrounds * npairs);
-  L.rrnd = take(sizeof(int) * 2 * nrounds);
+  L.escr = take(wide ? wide_eig_scr_bytes(T) : 1);
   L.wtc = take(wtc_bytes ? wtc_bytes : 1);
   L.gram_part = take(sizeof(float) * (size_t)maxgrid * T * T);
   L.group_part = take(sizeof(float2) * (size_t)L.ngroups * T * T);
@@ -214,7 +205,6 @@ struct rpca_plan_s {
   char* ws;
   bool own_ws;
   double lambda;
-  int eig_fp32;       // opt-in FP32 rotations in the narrow eigen-step (RPCA_EIG_FP32=1)
   cudaGraph_t graph;
   cudaGraphExec_t exec;
   Ctrl* ctrl_host;  // pinned
@@ -269,22 +259,21 @@ static cudaError_t launch(void* fn, dim3 g, dim3 blk, void** args, cudaStream_t 
   return cudaLaunchKernel(fn, g, blk, args, smem, s);
 }
 
-// Eigen-step kernel of a plan: FP64 Jacobi rotations and basis arithmetic,
-// or FP32 ones when RPCA_EIG_FP32 is set.  Both take (Bufs, flags, handle,
-// use_cond, ...); the extra pointer arguments of the argument lists below
-// are ignored.
+// Eigen-step kernel of a plan: (Bufs, flags, handle, use_cond) and, for wide
+// windows, its floats of shared memory.
 static void* eig_fn(const rpca_plan_s* pl) {
   if (pl->wide) return pl->wk.eig;
-  return pl->eig_fp32 ? pl->ks.eig_fast32 : pl->ks.eig_fast;
+  return pl->ks.eig_step;
 }
 static size_t eig_smem(const rpca_plan_s* pl) {
   if (pl->wide) return pl->wk.eig_smem;
-  return pl->eig_fp32 ? pl->ks.eig_fast32_smem : pl->ks.eig_fast_smem;
+  return pl->ks.eig_step_smem;
 }
 static dim3 eig_block(const rpca_plan_s* pl) {
   if (pl->wide) return dim3(pl->wk.eig_threads);
   return dim3(kEigThreads);
 }
+static dim3 eig_grid(const rpca_plan_s* pl) { return dim3(pl->wide ? pl->wk.eig_ctas : 1); }
 // CUDA-core FP32 passes by mode (narrow: one pixel row per thread, TMA-fed when
 // the plan has tensor maps; wide: tiles).
 static void* pass_fn(const rpca_plan_s* pl, int mode) {
@@ -344,23 +333,22 @@ static rpca_status build_graph(rpca_plan_s* pl) {
   cudaGraphConditionalHandle h;
   CK(cudaGraphConditionalHandleCreate(&h, pl->graph, 0, cudaGraphCondAssignDefault));
   Bufs b = pl->bufs;
-  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg(1), eb = eig_block(pl);
+  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg = eig_grid(pl), eb = eig_block(pl);
   const size_t es = eig_smem(pl);
-  const double* nulld = nullptr;
-  double* nullo = nullptr;
+  int eig_floats = (int)(eig_smem(pl) / sizeof(float));
   int use_cond = 1;
   int f_init = EF_INIT | EF_EIG, f_iter = EF_CHECK | EF_EIG;
 
   void* a_pass[] = {&b};
-  void* a_eig0[] = {&b, &f_init, &h, &use_cond, &nulld, &nullo, &nullo};
-  void* a_eig1[] = {&b, &f_iter, &h, &use_cond, &nulld, &nullo, &nullo};
+  void* a_eig0[] = {&b, &f_init, &h, &use_cond, &eig_floats};
+  void* a_eig1[] = {&b, &f_iter, &h, &use_cond, &eig_floats};
   cudaGraphNode_t n_init, n_eig0, n_while, n_fin, n_pass, n_eig;
   CK(add_kernel(pl->graph, &n_init, nullptr, 0, pass_fn(pl, PM_INIT), pg, pb, a_pass, pass_smem(pl)));
   CK(add_kernel(pl->graph, &n_eig0, &n_init, 1, eig_fn(pl), eg, eb, a_eig0, es));
   if (pl->p.warm_start) {
     // warm start: the first SVT needs the Gram of Z1 = X - S0 + Y0/mu1, not of X
     int f_eig = EF_EIG | EF_FULL;
-    void* a_eigw[] = {&b, &f_eig, &h, &use_cond, &nulld, &nullo, &nullo};
+    void* a_eigw[] = {&b, &f_eig, &h, &use_cond, &eig_floats};
     cudaGraphNode_t n_gw, n_ew;
     CK(add_kernel(pl->graph, &n_gw, &n_eig0, 1, pass_fn(pl, PM_GRAM), pg, pb, a_pass, pass_smem(pl)));
     CK(add_kernel(pl->graph, &n_ew, &n_gw, 1, eig_fn(pl), eg, eb, a_eigw, es));
@@ -393,7 +381,7 @@ void result_from_ctrl(double lambda, const Ctrl& c, rpca_result* out, int cplx) 
   out->iters = c.k;
   out->rank = cplx ? c.rank / 2 : c.rank;
   out->sweeps = c.total_sweeps;
-  out->resid = c.resid;
+  out->resid = c.k > 0 ? sqrt(c.res2) / c.normX : 0.0;
   out->mu = c.mu_cur;
   out->normX = c.normX;
   out->lambda = lambda;
@@ -534,17 +522,13 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   }
   pl->lay = make_layout(p->m, Tr, sms, pl->wide, pl->wide ? wide_tc_img_bytes(Tr, p->precision) : 0);
   if (!pl->wide) {
-    cudaError_t ea = cudaFuncSetAttribute(pl->ks.eig_fast, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)pl->ks.eig_fast_smem);
-    if (ea == cudaSuccess)
-      ea = cudaFuncSetAttribute(pl->ks.eig_fast32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)pl->ks.eig_fast32_smem);
+    cudaError_t ea = cudaFuncSetAttribute(pl->ks.eig_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)pl->ks.eig_step_smem);
     if (ea != cudaSuccess) {
       delete pl;
       return cuda_status(ea);
     }
   }
-  pl->eig_fp32 = (getenv("RPCA_EIG_FP32") && atoi(getenv("RPCA_EIG_FP32")) != 0) ? 1 : 0;
   if (workspace) {
     if (workspace_bytes < pl->lay.total || ((uintptr_t)workspace & 255u)) {
       delete pl;
@@ -573,9 +557,7 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   b.Ww = (float*)(pl->ws + pl->lay.ww);
   b.Vw = (float*)(pl->ws + pl->lay.vw);
   b.evw = (double*)(pl->ws + pl->lay.evw);
-  b.rot_log = (float2*)(pl->ws + pl->lay.rlog);
-  b.rot_k = (int*)(pl->ws + pl->lay.rk);
-  b.rot_rnd = (int*)(pl->ws + pl->lay.rrnd);
+  b.eig_scr = (float*)(pl->ws + pl->lay.escr);
   b.wtc = (pl->wide && p->precision == RPCA_PREC_TF32X3) ? 1 : (pl->wide && p->precision == RPCA_PREC_BF16X3) ? 2 : 0;
   b.wtc_img = b.wtc ? (unsigned char*)(pl->ws + pl->lay.wtc) : nullptr;
   b.m = p->m;
@@ -587,7 +569,6 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   // a sharded plan's passes finish their reduction themselves, so the summed
   // Gram and residual sums sit in the reduction record between the steps
   b.finalize = p->sharded ? 1 : 0;
-  b.eig64 = pl->wide ? 0 : (pl->eig_fp32 ? 0 : 1);
 
   const int mT = (int)std::max<int64_t>(p->m, p->T);
   pl->lambda = p->lambda > 0 ? p->lambda : 1.0 / sqrt((double)mT);
@@ -600,11 +581,6 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   c.mu0_scale = p->mu0_scale;
   c.mu_max_factor = p->mu_max_factor;
   c.tol = p->tol;
-  // Jacobi threshold: an off-diagonal pair rotates while |g_pq| > eps sqrt(g_pp g_qq);
-  // FP64 rotations stop 1e2 below the FP32 rounding of the passes' Gram entries
-  c.jacobi_eps = (b.eig64 ? 1e-9 : 1e-6);
-  c.warm_sweeps = 4;
-  c.cold_sweeps = 30;
   c.warm = p->warm_start;
   c.mu_init = p->mu_init;
   c.mu_prev_scale = p->mu_prev_scale;
@@ -642,22 +618,21 @@ extern "C" {
 // host after every iteration (one host synchronisation per iteration).
 static rpca_status run_host_loop(rpca_plan_s* pl, cudaStream_t s) {
   Bufs b = pl->bufs;
-  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg(1), eb = eig_block(pl);
+  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg = eig_grid(pl), eb = eig_block(pl);
   const size_t es = eig_smem(pl);
   cudaGraphConditionalHandle h = 0;
-  const double* nulld = nullptr;
-  double* nullo = nullptr;
+  int eig_floats = (int)(eig_smem(pl) / sizeof(float));
   int use_cond = 0;
   int f_init = EF_INIT | EF_EIG, f_check = EF_CHECK, f_eig = EF_EIG;
   void* a_pass[] = {&b};
-  void* a_init[] = {&b, &f_init, &h, &use_cond, &nulld, &nullo, &nullo};
-  void* a_check[] = {&b, &f_check, &h, &use_cond, &nulld, &nullo, &nullo};
-  void* a_eig[] = {&b, &f_eig, &h, &use_cond, &nulld, &nullo, &nullo};
+  void* a_init[] = {&b, &f_init, &h, &use_cond, &eig_floats};
+  void* a_check[] = {&b, &f_check, &h, &use_cond, &eig_floats};
+  void* a_eig[] = {&b, &f_eig, &h, &use_cond, &eig_floats};
   CK(launch(pass_fn(pl, PM_INIT), pg, pb, a_pass, s, pass_smem(pl)));
   CK(launch(eig_fn(pl), eg, eb, a_init, s, es));
   if (pl->p.warm_start) {
     int f_full = EF_EIG | EF_FULL;
-    void* a_full[] = {&b, &f_full, &h, &use_cond, &nulld, &nullo, &nullo};
+    void* a_full[] = {&b, &f_full, &h, &use_cond, &eig_floats};
     CK(launch(pass_fn(pl, PM_GRAM), pg, pb, a_pass, s, pass_smem(pl)));
     CK(launch(eig_fn(pl), eg, eb, a_full, s, es));
   }
@@ -683,21 +658,20 @@ static rpca_status run_host_loop(rpca_plan_s* pl, cudaStream_t s) {
 // at once.
 static rpca_status run_stream_loop(rpca_plan_s* pl, cudaStream_t s) {
   Bufs b = pl->bufs;
-  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg(1), eb = eig_block(pl);
+  const dim3 pg = pass_grid(pl), pb = pass_block(pl), eg = eig_grid(pl), eb = eig_block(pl);
   const size_t es = eig_smem(pl);
   cudaGraphConditionalHandle h = 0;
-  const double* nulld = nullptr;
-  double* nullo = nullptr;
+  int eig_floats = (int)(eig_smem(pl) / sizeof(float));
   int use_cond = 0;
   int f_init = EF_INIT | EF_EIG, f_iter = EF_CHECK | EF_EIG;
   void* a_pass[] = {&b};
-  void* a_init[] = {&b, &f_init, &h, &use_cond, &nulld, &nullo, &nullo};
-  void* a_iter[] = {&b, &f_iter, &h, &use_cond, &nulld, &nullo, &nullo};
+  void* a_init[] = {&b, &f_init, &h, &use_cond, &eig_floats};
+  void* a_iter[] = {&b, &f_iter, &h, &use_cond, &eig_floats};
   CK(launch(pass_fn(pl, PM_INIT), pg, pb, a_pass, s, pass_smem(pl)));
   CK(launch(eig_fn(pl), eg, eb, a_init, s, es));
   if (pl->p.warm_start) {
     int f_eig = EF_EIG | EF_FULL;
-    void* a_eig[] = {&b, &f_eig, &h, &use_cond, &nulld, &nullo, &nullo};
+    void* a_eig[] = {&b, &f_eig, &h, &use_cond, &eig_floats};
     CK(launch(pass_fn(pl, PM_GRAM), pg, pb, a_pass, s, pass_smem(pl)));
     CK(launch(eig_fn(pl), eg, eb, a_eig, s, es));
   }
@@ -898,13 +872,10 @@ rpca_status rpca_eig(const double* G, int32_t T, double* evals, double* evecs, v
   if (st != RPCA_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   Bufs b = pl->bufs;
-  int flags = EF_RAW;
-  cudaGraphConditionalHandle h = 0;
-  int use_cond = 0;
   double *ev = nullptr, *vv = nullptr;
   cudaError_t e = cudaMalloc(&ev, sizeof(double) * T);
   if (e == cudaSuccess) e = cudaMalloc(&vv, sizeof(double) * T * T);
-  void* args[] = {&b, &flags, &h, &use_cond, (void*)&G, &vv, &ev};
+  void* args[] = {&b, (void*)&G, &vv, &ev};
   if (e == cudaSuccess) e = launch(pl->ks.eig64, dim3(1), dim3(pl->ks.eig_threads), args, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   std::vector<double> evh(T), vvh((size_t)T * T), evs(T), vvs((size_t)T * T);
@@ -964,26 +935,25 @@ rpca_status rpca_step_run(rpca_plan_t pl, int32_t step, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   Bufs b = pl->bufs;
   cudaGraphConditionalHandle h = 0;
-  const double* nulld = nullptr;
-  double* nullo = nullptr;
+  int eig_floats = (int)(eig_smem(pl) / sizeof(float));
   int use_cond = 0;
   int flags = 0;
   void* a_pass[] = {&b};
-  void* a_eig[] = {&b, &flags, &h, &use_cond, &nulld, &nullo, &nullo};
+  void* a_eig[] = {&b, &flags, &h, &use_cond, &eig_floats};
   switch (step) {
     case RPCA_STEP_INIT:
       CK(launch(pass_fn(pl, PM_INIT), pass_grid(pl), pass_block(pl), a_pass, s, pass_smem(pl)));
       return RPCA_OK;
     case RPCA_STEP_EIG_INIT:
       flags = EF_INIT | EF_EIG;
-      CK(launch(eig_fn(pl), dim3(1), eig_block(pl), a_eig, s, eig_smem(pl)));
+      CK(launch(eig_fn(pl), eig_grid(pl), eig_block(pl), a_eig, s, eig_smem(pl)));
       return RPCA_OK;
     case RPCA_STEP_PASS:
       CK(launch(fused_fn(pl), fused_grid(pl), fused_block(pl), a_pass, s, fused_smem(pl)));
       return RPCA_OK;
     case RPCA_STEP_EIG:
       flags = EF_CHECK | EF_EIG;
-      CK(launch(eig_fn(pl), dim3(1), eig_block(pl), a_eig, s, eig_smem(pl)));
+      CK(launch(eig_fn(pl), eig_grid(pl), eig_block(pl), a_eig, s, eig_smem(pl)));
       return RPCA_OK;
     case RPCA_STEP_FINAL: {
       const int fgrid = (int)std::min<int64_t>((pl->p.m + 255) / 256, 4096);

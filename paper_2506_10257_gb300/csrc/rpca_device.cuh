@@ -26,7 +26,6 @@ namespace rpca {
 
 constexpr int kMaxT = 32;            // largest frame count of the register-resident passes
 constexpr int kMaxTW = 224;          // largest frame count of the wide (shared-memory tiled) path
-constexpr int kWideLogSweeps = 30;   // Jacobi sweeps one wide eigen-step may take (and log)
 constexpr int kPassThreads = 256;    // one pixel per thread per tile
 constexpr int kTile = kPassThreads;  // pixels per CTA tile
 constexpr int kPassCtasPerSm = 1;    // resident CTAs of the narrow passes per SM
@@ -51,6 +50,9 @@ struct Ctrl {
   int schedule;      // 0 IALM, 1 FIXED_L1
   double mu_cur;     // mu of the next pass (iteration k+1)
   double mu_nxt;     // mu of iteration k+2 (forms Z' in the fused pass)
+  double inv_cur;    // 1 / mu_cur
+  double inv_nxt;    // 1 / mu_nxt
+  double lim2;       // (tol ||X||_F)^2
   double mu_max;
   double lambda;
   double rho;
@@ -60,10 +62,7 @@ struct Ctrl {
   double normX2;     // ||X||_F^2
   double normX;      // ||X||_F
   double normX1;     // sum |X_ij|
-  double resid;      // relative residual of iteration k
-  double jacobi_eps; // graded off-diagonal threshold of the Jacobi sweeps
-  int warm_sweeps;   // sweep cap once warm started
-  int cold_sweeps;   // sweep cap of the first eigensolve
+  double res2;       // squared residual of iteration k (the host forms ||E||_F / ||X||_F from it)
   int warm;          // 1: the solve starts from S0 (in S) and Y0 (in the L buffer)
   int pad_w;
   double mu_init;       // > 0: first mu of the solve instead of the schedule's
@@ -146,7 +145,6 @@ struct Bufs {
   int wide;            // tiled path: the reduced Gram goes to Gw (T x T), else to red->G (kMaxT stride)
   int finalize;        // 1: the pass itself sums the group partials into red->G, e2, l1;
                        // 0: the next eigen-step does (saves a serial reduction level)
-  int eig64;           // narrow eigen-step: 1 FP64 Jacobi rotations and basis arithmetic, 0 FP32
   // T > kMaxT ("wide" windows): the reduced Gram, Wbar and V live in these
   // T x T row-major arrays of the workspace instead of red->G and EigState.
   double* Gw;          // summed partial Grams as FP64 (also scratch of the eigen-step)
@@ -155,9 +153,7 @@ struct Bufs {
   double* evw;
   unsigned char* wtc_img;  // tiled tensor-core pass: B operand images of Wbar and V (NULL: unused)
   int wtc;            // their arithmetic: 0 none, 1 TF32x3, 2 BF16x3
-  float2* rot_log;    // wide eigen-step: (c, s) of every rotated pair of every executed round
-  int* rot_k;         // ... its columns p | q << 8, bit 16 set on the first rotation of a round
-  int* rot_rnd;       // ... per round: round number and rotated pairs
+  float* eig_scr;     // wide eigen-step: its T x T operands, among them the transposed basis (EigScr)
 };
 
 }  // namespace rpca

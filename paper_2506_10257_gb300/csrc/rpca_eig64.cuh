@@ -1,309 +1,361 @@
-// rpca_eig64.cuh -- the narrow eigen-step (T <= 32) with FP64 Jacobi
-// rotations and FP64 basis arithmetic (included inside namespace rpca by
-// rpca_kernels.cuh).  This is the plans' default eigen-step.
+// rpca_eig64.cuh -- the narrow eigen-step (T <= 32): from the reduced Gram of
+// the rotated Z to Wbar and the next basis, to well beyond FP32 (included inside
+// namespace rpca by rpca_kernels.cuh).  One CTA of kEigThreads threads.
 //
-// Same iteration as eig_fast_body (cyclic Jacobi in round-robin order on the
-// rotated Gram G~ = V^T Z^T Z V, which arrives as FP64 sums of the CTAs' FP32
-// partials and nearly diagonal), arranged for GB300's FP64 pipe, where one
-// FP64 warp instruction occupies an SM sub-partition for tens of cycles: the
-// number of dependent FP64 instructions per round, not the flops, sets the
-// time.  So
-//   * a rotation's tangent t (GVL sym.schur2) is found in FP32, and (c, s) are
-//     then made orthonormal in FP64 (c^2 + s^2 = 1 + d, |d| ~ 1e-7, scaled by
-//     1 - d/2 + 3d^2/8): every rotation applied to G and V is an exact FP64
-//     orthogonal transform; the pair it targets is left with an off-diagonal
-//     entry ~1e-7 of its old value (computed, not assumed zero), which the
-//     next sweep removes;
-//   * every entry of J^T G J is computed from four entries of G in FP64 by one
-//     thread per upper-triangle entry, diagonal and targeted pair included
-//     (entries of two unrotated pairs are copied);
-//   * the rotations are applied to the columns of V (in shared memory, FP64,
-//     starting from the FP32 basis the pass used, exact in FP64) in the same
-//     round by the same threads, so no rotation log is replayed afterwards;
-//   * the entries a round's successor needs ((p,p), (q,q), (p,q) of each of
-//     its pairs) are computed from the current G by three lanes per pair of
-//     the last warp(s) while the other warps update the round, and one lane
-//     per pair forms the next rotation, so a round costs one CTA barrier.
-// After the sweeps V <- V (3I - V^T V)/2 (Newton-Schulz, FP64; to first order
-// it also removes the departure of the FP32-rounded old basis from
-// orthonormality), sigma = sqrt(lambda), the sigma > tau = 1/mu decision,
-// g = min(1, tau/sigma) and Wbar = V diag(g) V^T are FP64; Wbar and V are
-// rounded to FP32 once for the passes (Eq. 4 through the Gram).
+// GB300 runs FP64 at about 1/64 of its FP32 rate, so FP64 Jacobi sweeps bound
+// this step (262144 x 20: 105 us, of which 83 us sweeps; x 29: 310 us).  Here the
+// sweeps run in FP32 (rpca_jacobi.cuh) and only propose the eigenvectors U; what
+// the iteration uses is then formed from the Gram G and the basis V by products
+// whose sums are carried as two-float (hi, lo) pairs (Dot2 of Ogita, Rump and
+// Oishi, "Accurate sum and dot product", 2005: about 2^-46 of the terms) on the
+// FP32 pipe:
+//   Vn = V U,  Omega = Vn^T Vn - I,  H = G U,  Gp = U^T H   (= Vn^T (Z^T Z) Vn)
+// Omega is what U and the FP32-rounded V lack in orthonormality.  The larger
+// eigenvalue's vector keeps its direction: P = Vn (I - C), C_pq = Omega_pq for the
+// larger p, Omega_pp / 2 on the diagonal, so to first order
+//   P^T (Z^T Z) P = diag(d) + E,  d_p = Gp_pp (1 - Omega_pp),
+//                                 E_pq = Gp_pq - max(d_p, d_q) Omega_pq.
+// Wbar = f(Z^T Z) with f(sigma^2) = min(1, tau / sigma) is then
+//   I - P (diag(1 - g) - F o E) P^T,  F the divided differences of f
+// (g_divided_difference), right to second order in E and Omega; only the vectors
+// with sigma > tau enter it, so the others need not be separated from one another
+// and the sweeps stop once what is neglected on the former is below the result's
+// FP32 rounding.  A step that finds more left there runs another round of sweeps
+// on diag(d) + E.  sigma, the sigma > tau decision, g and mu are FP64.  Measured on
+// the windows above: 30 us (load 3, factor and sweeps 18, products and decisions 9)
+// and 52 us, at the same errors of L and S against 64 bits (1.0e-7 and 2.3e-7).
 #pragma once
 
-// Thread roles (8 warps; warp w runs on SM sub-partition w % 4): warp 7 forms
-// the rotations and is the only warp of its sub-partition with FP64 work, so
-// its dependent chain does not queue behind the updates; warps 0-2 and 4-6
-// update G and V; warp 3 waits at the barriers.
-template <int TB>
-struct Eig64Shape {
-  static constexpr int K = TB / 2;                          // pairs per round
-  static constexpr int NR = TB - 1;                         // rounds per sweep
-  static constexpr int NE = TB * (TB + 1) / 2;              // upper-triangle entries
-  static constexpr int LPP = K <= 10 ? 3 : 2;               // rotation lanes per pair
-  static constexpr int NW = 192;                            // threads updating G and V
-  static constexpr int EPT = (NE + NW - 1) / NW;            // entries per updating thread
-  static constexpr int VPT = (TB * K + NW - 1) / NW;        // (row, pair) items of V per updating thread
-  static_assert(LPP * K <= 32, "the rotation lanes exceed a warp");
-  static_assert(kEigThreads == 256, "eight warps");
-};
+constexpr int kEigThreads = 256;   // threads of the eigen-step CTA
+constexpr int kEigPasses = 3;      // rounds of sweeps one eigen-step may take
+constexpr float kEigStop = 3e-3f;  // largest cosine a sweep may meet and be the last
+constexpr float kEigInitStop = 1e-5f;  // ... of the first eigen-step, whose largest eigenvalue sets mu
+constexpr float kEigMaxOff = 4e-4f;    // largest |E_pq| corrected to first order, relative to sigma_p sigma_q where
+                                       // both enter Wbar, else to the larger sigma^2: what is neglected, 3/8 of
+                                       // its square, is FP32's rounding
+constexpr float kEigMaxOm = 2.4e-4f;    // largest |Omega_pq| (its square is neglected)
+constexpr float kEigNear = 0.25f;       // a sweep's cosines count where the longer column's sigma^2 / tau^2 is above this
 
-template <int TB>
 struct Eig64Smem {
-  double G[2][TB * (TB + 1)];
-  double V[TB * (TB + 1)];
-  double A[TB * (TB + 1)];
-  double2 cs[2][TB / 2];       // (c, s) of the current round and of the next (by round parity)
-  int2 pq[TB - 1][TB / 2];    // (p, q), p < q, of every pair of every round
-  int2 pinfo[TB - 1][TB];     // (pair index, slot) of every index in every round
-  double ev[TB];
-  double g[TB];
+  static constexpr int LD = kMaxT + 1;
+  static constexpr int N = kMaxT * LD;
+  float W[jac_floats(kMaxT)];         // columns of the Cholesky factor, then of L Q
+  float Gh[N], Gl[N];                 // G (scaled), columns and rows in descending order of the diagonal
+  float Vh[N], Vl[N];                 // the basis, columns in that order; then P
+  float U[N];
+  float Nh[N], Nl[N];                 // Vn; then K = P (diag(1 - g) - F o E)
+  float Hh[N], Hl[N];                 // H
+  float Om[N], E[N], C[N], B[N];
+  double d[kMaxT];
+  float sig[kMaxT], gh[kMaxT], gl[kMaxT] /* 1 - g */, diag[kMaxT], piv[kMaxT], nrm[kMaxT];
+  int perm[kMaxT], keep[kMaxT];
+  unsigned smax[2];
 };
 
-template <int TB>
-__device__ void eig64_body(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond, unsigned char* dsm) {
-  using SH = Eig64Shape<TB>;
-  constexpr int K = SH::K, NR = SH::NR, NE = SH::NE, NW = SH::NW, LPP = SH::LPP;
-  constexpr int LD = TB + 1;
-  Eig64Smem<TB>& S = *reinterpret_cast<Eig64Smem<TB>*>(dsm);
-  __shared__ int sFlag;
+// Dot2: (s, c) += a b, with the rounding errors of the product and of the sum in c.
+__device__ __forceinline__ void dot2(float& s, float& c, float a, float b) {
+  const float p = __fmul_rn(a, b);
+  const float e = fmaf(a, b, -p);
+  const float t = __fadd_rn(s, p);
+  const float z = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)), e));
+  s = t;
+}
+// (h, l) = s + c, normalised
+__device__ __forceinline__ void fast_two_sum(float s, float c, float& h, float& l) {
+  h = __fadd_rn(s, c);
+  l = __fsub_rn(c, __fsub_rn(h, s));
+}
+
+static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond,
+                                               unsigned char* dsm) {
+  Eig64Smem& S = *reinterpret_cast<Eig64Smem*>(dsm);
+  constexpr int LD = Eig64Smem::LD;
+  __shared__ EigCtl sCtl;
   __shared__ double sTau;
 
   Ctrl* ctrl = b.ctrl;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int T = b.T;
+  const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
+  const int T = b.T, TT = T * T;
+  const int JL = jac_ld(T), nb = jac_blocks(T);
   const unsigned long long t0 = gtimer();
-  if (!eig_control(b, flags, h, use_cond, &sFlag)) return;
-  const bool cold = (flags & EF_INIT) != 0;
+  const bool init = (flags & EF_INIT) != 0;
 
-  for (int i = tid; i < TB * TB; i += nthr) {
-    const int r = i / TB, c = i % TB;
-    const bool in = r < T && c < T;
-    S.G[0][r * LD + c] = in ? b.red->G[r * kMaxT + c] : 0.0;
-    double v = (r == c) ? 1.0 : 0.0;
-    if (!cold && in) v = (double)b.eig->V32[r * kMaxT + c];
-    S.V[r * LD + c] = v;
+  // T x T arrays: row = warp, warp + 8, ..., column = lane.  Upper triangles: entries
+  // (ep, eq) of this thread (at most ceil(528 / 256) = 3).
+  const int NE = T * (T + 1) / 2;
+  int ep[3], eq[3];
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    int e = tid + u * nthr, p = 0;
+    const bool in = e < NE;
+    if (in) tri_coords(e, T, p, e);
+    ep[u] = in ? p : -1;
+    eq[u] = e;
   }
-  for (int i = tid; i < NR * K; i += nthr) {
-    const int r = i / K, k = i % K;
-    int pa, pb;
-    rr_pair(r, k, TB, pa, pb);
-    const int p = min(pa, pb), q = max(pa, pb);
-    S.pq[r][k] = make_int2(p, q);
-    S.pinfo[r][p] = make_int2(k, 0);
-    S.pinfo[r][q] = make_int2(k, 1);
+
+  // the basis (its loads overlap the control part's)
+  float v0[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = warp + u * nwarps;
+    v0[u] = init ? (r == lane ? 1.f : 0.f) : (r < T && lane < T) ? __ldcg(&b.eig->V32[r * kMaxT + lane]) : 0.f;
   }
+  const bool go = eig_control(b, flags, h, use_cond, &sCtl, [&](int i0, int n) {
+    if (b.finalize) {
+      for (int i = i0; i < TT; i += n) {
+        const int r = i / T, c = i % T;
+        const double x = __ldcg(&b.red->G[r * kMaxT + c]);
+        const float xh = (float)x;
+        S.Hh[r * LD + c] = xh;
+        S.Hl[r * LD + c] = (float)(x - (double)xh);
+      }
+    } else {
+      sum_rows(b.group_part, 0, __ldcg(&b.red->ngroups_last), TT, [&](int e, float gh, float gl) {
+        S.Hh[e / T * LD + e % T] = gh;
+        S.Hl[e / T * LD + e % T] = gl;
+      }, i0, n);
+    }
+  });
+  if (!go) {
+    if (tid == nthr - 1) eig_control_tail(b, &sCtl);
+    return;
+  }
+
+  // ---- the Gram scaled by a power of four to about 1; the basis ----
+  const int pw = even_exponent(T <= 32 && lane < T ? S.Hh[lane * LD + lane] : 0.f);
+  const float scale = exp2i(-pw), rootf = exp2i(-pw / 2);
+  __syncthreads();
+  static_assert(kEigThreads / 32 * 4 >= kMaxT, "four rows a warp");
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = warp + u * nwarps;
+    if (r >= T || lane >= T) break;
+    S.Hh[r * LD + lane] *= scale;
+    S.Hl[r * LD + lane] *= scale;
+    S.Nh[r * LD + lane] = v0[u];
+    S.Nl[r * LD + lane] = 0.f;
+  }
+  if (tid < 2) S.smax[tid] = 0u;
+  if (tid == 0) sTau = sCtl.tau;
+  const double root = (double)rootf;
   __syncthreads();
   const unsigned long long t1 = gtimer();
-
-  const double eps = ctrl->jacobi_eps;
-  const double eps2 = eps * eps;
-  const float epsf2 = (float)eps2;
-  int max_sweeps = (cold || (flags & EF_FULL)) ? ctrl->cold_sweeps : ctrl->warm_sweeps;
-  if (max_sweeps > 30) max_sweeps = 30;
-  // roles (Eig64Shape): updating thread index wi in [0, NW) for warps 0-2 and
-  // 4-6; warp 7 forms the rotations, LPP lanes per pair
-  const int warp = tid >> 5;
-  const int wi = warp < 3 ? tid : (warp >= 4 && warp < 7 ? tid - 32 : -1);
-  const bool worker = wi >= 0;
-  const bool rwarp = warp == 7;
-  const int rl = tid & 31;                                          // lane
-  const int rk = (rwarp && rl < LPP * K) ? rl / LPP : K;            // pair of a rotation lane (K: none)
-  const int rj = rl % LPP;                                          // its part: 0 (p,p) [and (p,q) if LPP = 2],
-                                                                    // 1 (q,q), 2 (p,q)
-  const bool rlead = rwarp && rj == 0 && rk < K;
-  // The entries beyond the first NW (and the V items beyond the first NW) go
-  // to workers whose warps run on other sub-partitions than warp 0's, so
-  // the FP64 pipes of sub-partitions 0-2 carry about equal shares of a round.
-  int ea[SH::EPT], ec[SH::EPT];
+  unsigned long long t2 = t1, t3 = t1;
+  int sweeps = 0;
+  for (int pass = 0;; ++pass) {
+    // ---- descending order of the diagonal; Cholesky factor; one-sided Jacobi ----
+    // (every warp works the order out and writes the same values)
+    const float dl = lane < T ? S.Hh[lane * LD + lane] : 0.f;
+    int pos = 0;
+#pragma unroll 4
+    for (int j = 0; j < T; ++j) {
+      const float dj = S.Hh[j * LD + j];
+      pos += (int)(dj > dl) | ((int)(dj == dl) & (int)(j < lane));
+    }
+    if (lane < T) S.perm[pos] = lane;
+    __syncwarp();
+    auto perm = [&](int i) { return min((unsigned)S.perm[i < T ? i : 0], (unsigned)(T - 1)); };  // (in range for any values)
+    const int pl = perm(lane);
+    for (int c = warp; c < 4 * nb; c += nwarps) {
+      const int pc = perm(c);
+      if (lane < 16 * jac_r2(T)) S.W[c * JL + lane] = (lane < T && c <= lane) ? S.Hh[pl * LD + pc] : 0.f;
+      if (c < T && lane < T) {
+        const float gh = S.Hh[pc * LD + pl];
+        S.Gh[c * LD + lane] = gh;
+        S.Gl[c * LD + lane] = S.Hl[pc * LD + pl];
+        S.Vh[c * LD + lane] = S.Nh[c * LD + pl];
+        S.Vl[c * LD + lane] = S.Nl[c * LD + pl];
+        if (c == lane) S.diag[c] = gh;
+      }
+    }
+    __syncthreads();
+    jac_cholesky<1>(S.W, JL, T, S.diag, S.piv);
+    // the pairs that Wbar depends on: those with a singular value near or above tau
+    // (the first step's tau comes from its eigenvalues, a further pass wants them all)
+    const float taus = (float)(sTau * root);
+    const float lim = init || pass ? 0.f : fminf(kEigNear * taus * taus, 0.5f * S.diag[0]);
+    const float stop = init ? kEigInitStop : kEigStop;
+    const int cap = (init || (flags & EF_FULL)) ? 16 : 8;
+    sweeps += jac_r2(T) == 1 ? jac_sweeps<1>(S.W, JL, nb, S.nrm, S.smax, stop, lim, cap)
+                             : jac_sweeps<2>(S.W, JL, nb, S.nrm, S.smax, stop, lim, cap);
+    for (int c = warp; c < T; c += nwarps) {
+      const float x = lane < T ? S.W[c * JL + lane] : 0.f;
+      float n = x * x;
 #pragma unroll
-  for (int u = 0; u < SH::EPT; ++u) {
-    int e = (u == 0 ? wi : (wi + NW - 128) % NW) + u * NW, a = 0;
-    ea[u] = -1;
-    ec[u] = -1;
-    if (worker && e < NE) {
-      while (e >= TB - a) {
-        e -= TB - a;
-        ++a;
-      }
-      ea[u] = a;
-      ec[u] = a + e;
+      for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+      if (lane < T) S.U[lane * LD + c] = n > 0.f ? x * rsqrtf(n) : (lane == c ? 1.f : 0.f);
     }
-  }
-
-  // Entry (a, c) of J^T G J for round rnd's rotations in cs[cb] (G = S.G[cur]).
-  auto rot_entry = [&](int rnd, int cb, int cur, int a, int c) -> double {
-    const int2 ia = S.pinfo[rnd][a], ic = S.pinfo[rnd][c];
-    const double2 ra = S.cs[cb][ia.x], rc = S.cs[cb][ic.x];
-    if (ra.y == 0.0 && rc.y == 0.0) return S.G[cur][a * LD + c];
-    const int2 pa2 = S.pq[rnd][ia.x], pc2 = S.pq[rnd][ic.x];
-    // column a of J: slot 0 (c, -s) at (p, q); slot 1 (s, c)
-    const double wa0 = ia.y ? ra.y : ra.x, wa1 = ia.y ? ra.x : -ra.y;
-    const double wc0 = ic.y ? rc.y : rc.x, wc1 = ic.y ? rc.x : -rc.y;
-    const double* g0 = &S.G[cur][pa2.x * LD];
-    const double* g1 = &S.G[cur][pa2.y * LD];
-    const double u0 = fma(wc1, g0[pc2.y], wc0 * g0[pc2.x]);
-    const double u1 = fma(wc1, g1[pc2.y], wc0 * g1[pc2.x]);
-    return fma(wa1, u1, wa0 * u0);
-  };
-  // Rotation of a pair from (app, aqq, apq) into cs[cb][k]; returns whether it rotates.
-  // The threshold test and the tangent run on FP32 copies of the three
-  // entries (the test's outcome only decides whether the pair rotates this
-  // sweep; rotating or not, G stays an exact FP64 similarity transform of the
-  // Gram), so the FP64 part of the chain is the conversions and the
-  // normalisation.
-  auto make_rotation = [&](int cb, int k, double app, double aqq, double apq) -> int {
-    double c = 1.0, s = 0.0;
-    int act = 0;
-    const float apf = (float)apq, ppf = (float)app, qqf = (float)aqq;
-    if (apf != 0.f && apf * apf > epsf2 * fabsf(ppf * qqf)) {
-      act = 1;
-      const float ddf = qqf - ppf;
-      const float r2 = fmaf(ddf, ddf, 4.f * apf * apf);
-      const float tf = copysignf(1.f, ddf) * (2.f * apf) / (fabsf(ddf) + sqrtf(r2));
-      if (isfinite(tf) && isfinite(r2) && fabsf(apf) > 1e-30f) {
-        const float cf = rsqrtf(fmaf(tf, tf, 1.f));
-        c = (double)cf;
-        s = (double)(tf * cf);
-      } else {
-        // outside FP32 range: the same rotation in FP64
-        const double dd = aqq - app;
-        const double t = copysign(1.0, dd) * (2.0 * apq) / (fabs(dd) + sqrt(fma(dd, dd, 4.0 * apq * apq)));
-        c = 1.0 / sqrt(fma(t, t, 1.0));
-        s = t * c;
+    if (tid < 2) S.smax[tid] = 0u;
+    __syncthreads();
+    t2 = gtimer();
+    // ---- Vn = V U, H = G U ----
+#pragma unroll 1
+    for (int r = warp; r < T; r += nwarps) {
+      if (lane >= T) break;
+      const int c = lane;
+      float s = 0.f, e = 0.f, hs = 0.f, he = 0.f;
+#pragma unroll 2
+      for (int k = 0; k < T; ++k) {
+        const float u = S.U[k * LD + c];
+        dot2(s, e, S.Vh[r * LD + k], u);
+        e = fmaf(S.Vl[r * LD + k], u, e);
+        dot2(hs, he, S.Gh[r * LD + k], u);
+        he = fmaf(S.Gl[r * LD + k], u, he);
       }
-      // exact FP64 orthonormality: scale by (c^2 + s^2)^(-1/2) to third order
-      const double d = fma(c, c, s * s) - 1.0;
-      const double r = fma(fma(0.375, d, -0.5), d, 1.0);
-      c *= r;
-      s *= r;
+      fast_two_sum(s, e, S.Nh[r * LD + c], S.Nl[r * LD + c]);
+      fast_two_sum(hs, he, S.Hh[r * LD + c], S.Hl[r * LD + c]);
     }
-    S.cs[cb][k] = make_double2(c, s);
-    return act;
-  };
-
-  int cur = 0, sweeps = 0, rounds_run = 0;
-  while (sweeps < max_sweeps) {
-    int need = 0;
+    __syncthreads();
+    // ---- Omega = Vn^T Vn - I, Gp = U^T H (upper triangles; Gp stays in registers) ----
+    float gph[3], gpl[3];
 #pragma unroll
-    for (int u = 0; u < SH::EPT; ++u) {
-      const int a = ea[u], c = ec[u];
-      if (a >= 0 && a < c) {
-        const double apq = S.G[cur][a * LD + c];
-        if (apq != 0.0 && apq * apq > eps2 * fabs(S.G[cur][a * LD + a] * S.G[cur][c * LD + c])) need = 1;
+    for (int u = 0; u < 3; ++u) {
+      if (u * kEigThreads >= NE) break;
+      const int p = ep[u], q = eq[u];
+      if (p < 0) continue;
+      float s = p == q ? -1.f : 0.f, e = 0.f, gs = 0.f, ge = 0.f;
+#pragma unroll 2
+      for (int k = 0; k < T; ++k) {
+        const float ph = S.Nh[k * LD + p], qh = S.Nh[k * LD + q];
+        dot2(s, e, ph, qh);
+        e = fmaf(ph, S.Nl[k * LD + q], fmaf(S.Nl[k * LD + p], qh, e));
+        const float up = S.U[k * LD + p];
+        dot2(gs, ge, up, S.Hh[k * LD + q]);
+        ge = fmaf(up, S.Hl[k * LD + q], ge);
+      }
+      S.Om[p * LD + q] = __fadd_rn(s, e);
+      fast_two_sum(gs, ge, gph[u], gpl[u]);
+      if (p == q) {
+        const double gp = (double)gph[u] + (double)gpl[u];
+        S.d[p] = gp - gp * (double)S.Om[p * LD + p];
       }
     }
-    if (!__syncthreads_or(need)) break;
-    int act = 0;
-    if (rlead) {
-      const int2 pq = S.pq[0][rk];
-      act = make_rotation(0, rk, S.G[cur][pq.x * LD + pq.x], S.G[cur][pq.y * LD + pq.y], S.G[cur][pq.x * LD + pq.y]);
-    }
-    int any = __syncthreads_or(act);
-    for (int rnd = 0; rnd < NR; ++rnd) {
-      const int cb = rnd & 1;
-      const int nxt = any ? (cur ^ 1) : cur;
-      if (any && worker) {
-        ++rounds_run;
-#pragma unroll
-        for (int u = 0; u < SH::EPT; ++u) {
-          const int a = ea[u], c = ec[u];
-          if (a < 0) continue;
-          const double v = rot_entry(rnd, cb, cur, a, c);
-          S.G[nxt][a * LD + c] = v;
-          S.G[nxt][c * LD + a] = v;
-        }
-        // V <- V J on the round's pairs (each (row, pair) item touches only its two entries)
-#pragma unroll
-        for (int u = 0; u < SH::VPT; ++u) {
-          const int item = (u == 0 ? wi : (wi + NW - 64) % NW) + u * NW;
-          if (item >= T * K) continue;
-          const int r = item / K, k = item % K;
-          const double2 r2 = S.cs[cb][k];
-          if (r2.y == 0.0) continue;
-          const int2 pq = S.pq[rnd][k];
-          const double vp = S.V[r * LD + pq.x], vq = S.V[r * LD + pq.y];
-          S.V[r * LD + pq.x] = fma(r2.x, vp, -r2.y * vq);
-          S.V[r * LD + pq.y] = fma(r2.y, vp, r2.x * vq);
-        }
-      }
-      int act_next = 0;
-      if (rwarp && rnd + 1 < NR) {
-        // the entries (p,p), (q,q), (p,q) of the next round's pair rk after this
-        // round, LPP lanes per pair
-        double v = 0.0, w = 0.0;
-        if (rk < K) {
-          const int2 pq = S.pq[rnd + 1][rk];
-          const int a = rj == 1 ? pq.y : pq.x, c = rj == 0 ? pq.x : pq.y;
-          v = any ? rot_entry(rnd, cb, cur, a, c) : S.G[cur][a * LD + c];
-          if (LPP == 2 && rj == 0) w = any ? rot_entry(rnd, cb, cur, pq.x, pq.y) : S.G[cur][pq.x * LD + pq.y];
-        }
-        const unsigned full = 0xffffffffu;
-        const double aqq = __shfl_sync(full, v, rl + 1 < 32 ? rl + 1 : rl);
-        const double apq = LPP == 2 ? w : __shfl_sync(full, v, rl + 2 < 32 ? rl + 2 : rl);
-        if (rlead) act_next = make_rotation(cb ^ 1, rk, v, aqq, apq);
-      }
-      if (any) cur = nxt;
-      any = __syncthreads_or(act_next);
-    }
-    ++sweeps;
-  }
-
-  const unsigned long long t2 = gtimer();
-  if (tid < TB) S.ev[tid] = S.G[cur][tid * LD + tid];
-  const int qb = cur ^ 1;  // free buffer
-  // Newton-Schulz: A = 1.5 I - 0.5 V^T V (symmetric), then V <- V A -> S.G[qb]
-  for (int i = tid; i < TB * TB; i += nthr) {
-    const int a = i / TB, c = i % TB;
-    if (a > c) continue;
-    double acc = 0.0;
-    if (c < T)
-      for (int r = 0; r < T; ++r) acc = fma(S.V[r * LD + a], S.V[r * LD + c], acc);
-    const double v = (a == c ? 1.5 : 0.0) - 0.5 * acc;
-    S.A[a * LD + c] = v;
-    S.A[c * LD + a] = v;
-  }
-  __syncthreads();
-  for (int i = tid; i < TB * TB; i += nthr) {
-    const int r = i / TB, c = i % TB;
-    double acc = 0.0;
-    if (r < T && c < T)
-      for (int a = 0; a < T; ++a) acc = fma(S.V[r * LD + a], S.A[a * LD + c], acc);
-    S.G[qb][r * LD + c] = acc;
-  }
-  const unsigned long long t3 = gtimer();
-
-  // ---- FP64 decisions: mu (first call), tau, sigma > tau, g ----
-  if (tid == 0) {
-    if (flags & EF_INIT) {
+    __syncthreads();
+    // ---- FP64 decisions: mu (first call), tau, sigma > tau, g ----
+    if (init && tid == 0) {
       double lmax = 0.0;
-      for (int a = 0; a < T; ++a) lmax = fmax(lmax, S.ev[a]);
-      init_mu(b, lmax);
+      for (int a = 0; a < T; ++a) lmax = fmax(lmax, S.d[a]);
+      init_mu(b, lmax / (double)scale);
+      sTau = ctrl->inv_cur;
     }
-    sTau = 1.0 / ctrl->mu_cur;
+    if (init) __syncthreads();
+    if (tid < T) {
+      const double tau = sTau * root;
+      // 1 / sigma by one third-order (Halley) step from its FP32 value: a few FP64
+      // operations where a square root and a division would take tens
+      const double dv = S.d[tid];
+      const bool pos = dv > 1e-36;  // (scaled by the largest: below that it is rounding)
+      const double y0 = pos ? (double)rsqrtf((float)dv) : 0.0;
+      const double er = fma(-dv * y0, y0, 1.0);
+      const double y = fma(y0 * er, fma(er, 0.375, 0.5), y0);
+      const double sg = pos ? dv * y : 0.0;
+      const int keep = sg > tau;
+      const double g1 = keep ? fma(-tau, y, 1.0) : 0.0;
+      S.keep[tid] = keep;
+      S.sig[tid] = (float)sg;
+      S.gh[tid] = (float)g1;
+      S.gl[tid] = (float)(g1 - (double)(float)g1);
+    }
+    __syncthreads();
+    // ---- E, C and -F o E ----
+    const float tauf = (float)(sTau * root);
+    int more = 0;
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int p = ep[u], q = eq[u];
+      if (p < 0) continue;
+      const float om = S.Om[p * LD + q];
+      if (p == q) {
+        S.C[p * LD + p] = 0.5f * om;
+        S.E[p * LD + p] = 0.f;
+        S.B[p * LD + p] = 0.f;
+        continue;
+      }
+      const bool pbig = S.d[p] >= S.d[q];
+      const float dm = (float)(pbig ? S.d[p] : S.d[q]);
+      const float sp = fmaxf(S.sig[p], S.sig[q]), sq = fminf(S.sig[p], S.sig[q]);
+      const float ev = fmaf(-dm, om, gph[u]) + gpl[u];
+      S.C[p * LD + q] = pbig ? om : 0.f;
+      S.C[q * LD + p] = pbig ? 0.f : om;
+      S.E[p * LD + q] = ev;
+      S.E[q * LD + p] = ev;
+      const float bv = -g_divided_difference(sp, sq, tauf) * ev;
+      S.B[p * LD + q] = bv;
+      S.B[q * LD + p] = bv;
+    }
+    __syncthreads();
+    // ---- P = Vn (I - C); whether E is small enough.  Pairs of two singular values
+    //      below tau do not enter Wbar, unless what the sweeps left between them
+    //      could hide an eigenvalue above tau^2 (Gershgorin's bound of the row) ----
+#pragma unroll 1
+    for (int r = warp; r < T; r += nwarps) {
+      const int c = lane < T ? lane : 0;
+      float s = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < T; ++k) s = fmaf(S.Nh[r * LD + k], S.C[k * LD + c], s);
+      const float sr = S.sig[r], sc = S.sig[c], ev = fabsf(S.E[r * LD + c]);
+      const bool kept = S.keep[r] || S.keep[c], both = S.keep[r] && S.keep[c];
+      const float hi = fmaxf(sr, sc);
+      const bool off = lane < T && r != c && (ev > kEigMaxOff * hi * (both ? fminf(sr, sc) : hi) ||
+                                           fabsf(S.Om[min(r, c) * LD + max(r, c)]) > kEigMaxOm);
+      if (off && kept) more = 1;
+      float hid = off && !kept ? ev : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) hid += __shfl_xor_sync(0xffffffffu, hid, o);
+      if (hid > 0.f && !S.keep[r] && fmaf(sr, sr, hid) > tauf * tauf) more = 1;
+      if (lane < T) fast_two_sum(S.Nh[r * LD + c], S.Nl[r * LD + c] - s, S.Vh[r * LD + c], S.Vl[r * LD + c]);
+    }
+    more = __syncthreads_or(more);
+    if (!more || pass + 1 == kEigPasses) break;
+    // another round on diag(d) + E in the basis P
+#pragma unroll 1
+    for (int r = warp; r < T; r += nwarps) {
+      if (lane >= T) break;
+      const int c = lane;
+      const double x = r == c ? S.d[r] : (double)S.E[r * LD + c];
+      const float xh = (float)x;
+      S.Hh[r * LD + c] = xh;
+      S.Hl[r * LD + c] = (float)(x - (double)xh);
+      S.Nh[r * LD + c] = S.Vh[r * LD + c];
+      S.Nl[r * LD + c] = S.Vl[r * LD + c];
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  int keep = 0;
-  if (tid < TB) {
-    const double sig = sqrt(fmax(S.ev[tid], 0.0));
-    keep = (tid < T) && (sig > sTau);
-    S.g[tid] = keep ? sTau / sig : 1.0;
+  t3 = gtimer();
+  // ---- K = P (diag(1 - g) - F o E), then Wbar = I - K P^T (upper triangle, mirrored) ----
+  if (tid == nthr - 1) eig_control_tail(b, &sCtl);
+#pragma unroll 1
+  for (int r = warp; r < T; r += nwarps) {
+    if (lane >= T) break;
+    const int c = lane;
+    float s = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < T; ++k) s = fmaf(S.Vh[r * LD + k], S.B[k * LD + c], s);
+    const float ph = S.Vh[r * LD + c], gh = S.gh[c];
+    const float p = __fmul_rn(ph, gh);
+    const float e = fmaf(ph, gh, -p) + fmaf(ph, S.gl[c], S.Vl[r * LD + c] * gh);
+    fast_two_sum(p, e + s, S.Nh[r * LD + c], S.Nl[r * LD + c]);
+    b.eig->V32[r * kMaxT + c] = ph;  // (normalised: the pair rounded to FP32)
   }
-  const int rank = __syncthreads_count(keep);
-
-  // Wbar = V diag(g) V^T in FP64 (upper triangle, mirrored), rounded to FP32
-  // once; V rounded to FP32 for the next pass
-  const double* Vn = S.G[qb];
-  for (int i = tid; i < T * T; i += nthr) {
-    const int a = i / T, c = i % T;
-    b.eig->V32[a * kMaxT + c] = (float)Vn[a * LD + c];
-    if (a > c) continue;
-    double acc = 0.0;
-    for (int j = 0; j < T; ++j) acc = fma(Vn[a * LD + j] * S.g[j], Vn[c * LD + j], acc);
-    b.eig->Wbar[a * kMaxT + c] = (float)acc;
-    b.eig->Wbar[c * kMaxT + a] = (float)acc;
+  const int rank = __syncthreads_count(tid < T && S.keep[tid]);
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    const int p = ep[u], q = eq[u];
+    if (p < 0) continue;
+    float s = p == q ? -1.f : 0.f, e = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < T; ++k) {
+      const float kh = S.Nh[p * LD + k], ph = S.Vh[q * LD + k];
+      dot2(s, e, kh, ph);
+      e = fmaf(kh, S.Vl[q * LD + k], fmaf(S.Nl[p * LD + k], ph, e));
+    }
+    const float w = -(s + e);
+    b.eig->Wbar[p * kMaxT + q] = w;
+    b.eig->Wbar[q * kMaxT + p] = w;
   }
-  if (tid < T) b.eig->evals[tid] = S.ev[tid];
+  if (tid < T) b.eig->evals[tid] = S.d[tid] / (double)scale;
   if (tid == 0) {
     ctrl->rank = rank;
     ctrl->sweeps = sweeps;
@@ -315,14 +367,13 @@ __device__ void eig64_body(Bufs b, int flags, cudaGraphConditionalHandle h, int 
     ctrl->eig_phase_ns[1] += t2 - t1;
     ctrl->eig_phase_ns[2] += t3 - t2;
     ctrl->eig_phase_ns[3] += t4 - t3;
-    ctrl->eig_rounds += rounds_run;
+    ctrl->eig_rounds += sweeps * (nb - 1);
     set_cond(h, use_cond, 1u);
   }
 }
 
-template <int TB>
-__global__ void __launch_bounds__(kEigThreads) eig64_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,
-                                                            int use_cond) {
+static __global__ void __launch_bounds__(kEigThreads) eig64_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,
+                                                                   int use_cond) {
   extern __shared__ __align__(16) unsigned char eig64_smem_raw[];
-  eig64_body<TB>(b, flags, h, use_cond, eig64_smem_raw);
+  eig64_body(b, flags, h, use_cond, eig64_smem_raw);
 }

@@ -28,10 +28,14 @@ struct WideKernels {
   void* eig;            // (Bufs, flags, handle, use_cond)
   size_t eig_smem;
   int eig_threads;
+  int eig_ctas;
   void* pass_tc[4];     // fused pass on the tensor cores per rpca_precision (real TP <= 128; NULL: none)
   size_t pass_tc_smem[4];
   int pass_tc_threads;
 };
+
+// Bytes of a wide eigen-step's scratch for T real columns.
+size_t wide_eig_scr_bytes(int T);
 
 // Bytes of the B operand images a tiled tensor-core plan keeps (0: none).
 size_t wide_tc_img_bytes(int T, int precision);

@@ -37,13 +37,14 @@ __device__ __forceinline__ bool solve_done_uniform(const Ctrl* ctrl) {
 
 // Jacobi round-robin pairing (circle method) on n indices, round r in [0, n-1).
 __device__ __forceinline__ void rr_pair(int r, int i, int n, int& a, int& b) {
-  const int k = n - 1;
+  const int k = n - 1;  // (r < k, so the sums below wrap at most once)
   if (i == 0) {
     a = 0;
-    b = (r % k) + 1;
+    b = r + 1;
   } else {
-    a = ((r + i) % k) + 1;
-    b = ((r - i + k) % k) + 1;
+    const int u = r + i, v = r - i;
+    a = (u >= k ? u - k : u) + 1;
+    b = (v < 0 ? v + k : v) + 1;
   }
 }
 
@@ -183,18 +184,20 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float bh, float bl)
 __device__ __forceinline__ float2 ff_term(float v) { return make_float2(v, 0.f); }
 __device__ __forceinline__ float2 ff_term(float2 v) { return v; }
 
-// Sums rows [r0, r1) of a row-major [rows][TT] array (FP32 partials of the
+// Sums rows [r0, r1) of entries [e0, e1) (all by default) of a row-major [rows][TT] array (FP32 partials of the
 // CTAs, or two-float group sums) entry by entry in two-float arithmetic in a
 // fixed row order, calling out(e, hi, lo) for every entry; each thread takes
 // entries tid, tid + blockDim, ... and issues its loads in batches of 16 so
 // that their L2 latencies overlap.  The reduced Gram thus carries only the
 // rounding of the CTAs' own FP32 accumulations.
 template <int W = 1, typename Src, typename Out>
-__device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT, Out out) {
+__device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT, Out out, int tid = threadIdx.x,
+                                         int nthr = blockDim.x, int e0 = 0, int e1 = -1) {
   // W = 4: four entries per step (T x T Grams of wide windows), so that 64
   // loads are in flight per thread
-  int e = threadIdx.x;
-  for (; W == 4 && e + 3 * (int)blockDim.x < TT; e += 4 * blockDim.x) {
+  if (e1 < 0) e1 = TT;
+  int e = e0 + tid;
+  for (; W == 4 && e + 3 * nthr < e1; e += 4 * nthr) {
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
     for (int rb = r0; rb < r1; rb += 16) {
       Src v[4][16];
@@ -202,7 +205,7 @@ __device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT,
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int u = 0; u < 16; ++u)
-          v[q][u] = (rb + u < r1) ? __ldcg(&src[(int64_t)(rb + u) * TT + e + q * blockDim.x]) : Src{};
+          v[q][u] = (rb + u < r1) ? __ldcg(&src[(int64_t)(rb + u) * TT + e + q * nthr]) : Src{};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -212,9 +215,9 @@ __device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT,
         }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out(e + q * blockDim.x, h[q], l[q]);
+    for (int q = 0; q < 4; ++q) out(e + q * nthr, h[q], l[q]);
   }
-  for (; e < TT; e += blockDim.x) {
+  for (; e < e1; e += nthr) {
     float h = 0.f, l = 0.f;
     for (int rb = r0; rb < r1; rb += 16) {
       Src v[16];
@@ -468,6 +471,11 @@ __host__ __device__ constexpr size_t pass_simt_smem() {
 // per-thread group bookkeeping that orders it before this thread's reads.
 __device__ __forceinline__ void cp_async4(float* sdst, const float* gsrc) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(sdst)),
+               "l"(gsrc)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* sdst, const float* gsrc) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sdst)),
                "l"(gsrc)
                : "memory");
 }
@@ -785,25 +793,24 @@ __global__ void __launch_bounds__(kPassThreads, pass_min_blocks<TB>()) pass_kern
 // Iteration control + eigensolve, one CTA.
 //   EF_INIT  : ||X|| from the init pass; X == 0 finishes with L = S = 0
 //   EF_CHECK : residual test of the iteration just done (Sec. II-A), mu update
-//   EF_EIG   : cyclic Jacobi on the rotated Gram (warm start from V), then
+//   EF_EIG   : Jacobi on the rotated Gram (warm start from V), then
 //              sigma = sqrt(lambda), the sigma > tau decision and
 //              Wbar = V diag(min(1, tau/sigma)) V^T (FP64 decisions)
-//   EF_RAW   : decompose an external FP64 matrix only (kernel-level tests)
-// Real is the arithmetic of the Jacobi rotations (float or double).
 // ---------------------------------------------------------------------------
-enum { EF_RAW = 8 };
-
 __device__ __forceinline__ void set_cond(cudaGraphConditionalHandle h, int use, unsigned v) {
   if (use) cudaGraphSetConditional(h, v);
 }
 
+// FP32 copies of mu and its reciprocals for the passes; inv_cur = 1 / mu_cur.
 __device__ __forceinline__ void refresh_f32(Ctrl* c) {
-  // one FP64 division when mu_nxt = mu_cur (fixed or capped), else two
-  const double inv = 1.0 / c->mu_cur;
   c->f_mu = (float)c->mu_cur;
-  c->f_inv_mu = (float)inv;
-  c->f_gamma = (float)(c->lambda * inv);
-  c->f_inv_mu_nxt = (float)(c->mu_nxt == c->mu_cur ? inv : 1.0 / c->mu_nxt);
+  c->f_inv_mu = (float)c->inv_cur;
+  c->f_gamma = (float)(c->lambda * c->inv_cur);
+}
+__device__ __forceinline__ void refresh_next(Ctrl* c) {
+  const double inv = c->mu_nxt == c->mu_cur ? c->inv_cur : 1.0 / c->mu_nxt;
+  c->inv_nxt = inv;
+  c->f_inv_mu_nxt = (float)inv;
 }
 
 // First mu of a solve (FP64, thread 0 of an eigen-step with EF_INIT): the
@@ -825,142 +832,160 @@ __device__ __forceinline__ void init_mu(Bufs b, double lmax) {
   c->mu_max = c->mu_max_factor * mu0;
   c->mu_nxt = (c->schedule == 0) ? fmin(c->rho * mu1, c->mu_max) : mu1;
   c->k = 0;
+  c->inv_cur = 1.0 / mu1;
   refresh_f32(c);
+  refresh_next(c);
 }
 
-// Final sums of a pass that left them as group partials (finalize == 0):
-// red->G, red->e2, red->l1 from the group partials, fixed order.  All threads
-// of the calling CTA take part.
-static __device__ void finalize_sums(Bufs b, double* sh) {
-  if (b.finalize) return;
-  const int T = b.T, TT = T * T;
-  const int ng = b.red->ngroups_last;
-  if (b.red->gram_last) {
-    if (b.wide) {
-      double* G = b.Gw;
-      sum_rows<4>(b.group_part, 0, ng, TT, [&](int e, float h, float l) { G[e] = (double)h + (double)l; });
+// What the control part of an eigen-step leaves for the rest of it.
+struct EigCtl {
+  int stop;     // the solve ends here (or no eigensolve was asked for)
+  int tail;     // 1: 1 / mu_nxt is still to be computed (eig_control_tail)
+  double tau;   // 1 / mu of this step (0 in the first step, whose mu comes from its eigenvalues)
+};
+
+// Control part of an eigen-step, run by warp 0 alone while the other warps call
+// gram(i, n) (thread i of n) to sum the Gram of the pass that just ran: accounts
+// the pass's timing, sums its scalar partials, applies EF_CHECK (the residual
+// test of Sec. II-A after the iteration, in FP64 and without its square root and
+// division, then the mu update) and EF_INIT (||X|| from the init pass; X == 0
+// finishes with L = S = 0), and sets the graph's loop condition when the solve
+// ends here.  An FP64 division or square root takes about half a microsecond
+// here, so the residual is reported as its square and 1 / mu of the iteration
+// after the next, which nothing in this step waits for, is left to
+// eig_control_tail.  All threads call it; true: go on to the eigensolve.
+template <typename GramF>
+static __device__ __forceinline__ bool eig_control(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond,
+                                                   EigCtl* ec, GramF gram) {
+  Ctrl* c = b.ctrl;
+  RedState* red = b.red;
+  if ((threadIdx.x >> 5) != 0) {
+    gram((int)threadIdx.x - 32, (int)blockDim.x - 32);
+  } else {
+    const int lane = threadIdx.x;
+    // every load before the first store, so that their latencies overlap
+    const int was_done = __ldcg(&c->done), k0 = __ldcg(&c->k), err = __ldcg(&red->err);
+    const int max_iter = __ldcg(&c->max_iter), schedule = __ldcg(&c->schedule);
+    const double mu_nxt = __ldcg(&c->mu_nxt), inv_nxt = __ldcg(&c->inv_nxt), inv_cur = __ldcg(&c->inv_cur);
+    const double rho = __ldcg(&c->rho), mu_max = __ldcg(&c->mu_max), lim2 = __ldcg(&c->lim2);
+    const double lambda = __ldcg(&c->lambda), tol = __ldcg(&c->tol);
+    const unsigned long long ts = __ldcg(&red->t_start), te = __ldcg(&red->t_end);
+    const unsigned long long tl = __ldcg(&red->t_loop), t1 = __ldcg(&red->t_l1);
+    double e2 = 0.0, l1 = 0.0;
+    if (b.finalize) {
+      e2 = __ldcg(&red->e2);
+      l1 = __ldcg(&red->l1);
     } else {
-      double* G = b.red->G;
-      sum_rows(b.group_part, 0, ng, TT,
-               [&](int e, float h, float l) { G[(e / T) * kMaxT + e % T] = (double)h + (double)l; });
+      // (at most kMaxGroups = 64 rows; rows of groups that did not run are not read)
+      const int ng = __ldcg(&red->ngroups_last);
+      if (lane < ng) {
+        e2 = __ldcg(&b.gscal_part[2 * lane]);
+        l1 = __ldcg(&b.gscal_part[2 * lane + 1]);
+      }
+      if (lane + 32 < ng) {
+        e2 += __ldcg(&b.gscal_part[2 * (lane + 32)]);
+        l1 += __ldcg(&b.gscal_part[2 * (lane + 32) + 1]);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+        if (flags & EF_INIT) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+      }
     }
-  }
-  sum_scalars(b.gscal_part, 0, ng, sh, [&](double s0, double s1) {
-    b.red->e2 = s0;
-    b.red->l1 = s1;
-  });
-  __syncthreads();
-}
-
-// Control part of an eigen-step, shared by both eigen kernels (all threads call
-// it): accounts the timing of the pass that just ran, applies EF_CHECK (the
-// residual test of Sec. II-A after the iteration, then the mu update) and
-// EF_INIT (||X|| from the init pass; X == 0 finishes with L = S = 0), and sets
-// the graph's loop condition when the solve ends here.  Returns true when the
-// caller goes on to the eigensolve.
-static __device__ bool eig_control(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond, int* sFlag) {
-  Ctrl* ctrl = b.ctrl;
-  const int tid = threadIdx.x;
-  __shared__ double sFin[2 * kMaxGroups];
-  if (!ctrl->done) finalize_sums(b, sFin);
-  if (tid == 0) {
-    (*sFlag) = ctrl->done;
-    // account the pass that just ran (the first iteration's pass reads no S, Y
-    // and is left out of the steady-state average)
-    const unsigned long long ts = b.red->t_start, te = b.red->t_end;
-    const unsigned long long tl = b.red->t_loop, t1 = b.red->t_l1;
-    if (ts != ~0ull && te > ts) {
-      if (flags & EF_INIT) {
-        ctrl->init_ns = te - ts;
-      } else if ((flags & EF_CHECK) && ctrl->k >= 1) {
-        ctrl->pass_ns += te - ts;
-        ctrl->pass_cnt += 1;
-        if (tl >= ts && t1 >= tl && te >= t1) {
-          ctrl->pass_phase_ns[0] += tl - ts;
-          ctrl->pass_phase_ns[1] += t1 - tl;
-          ctrl->pass_phase_ns[2] += te - t1;
+    if (lane == 0) {
+      int stop = was_done, tail = 0;
+      double tau = inv_cur;
+      if (!stop && (flags & EF_CHECK)) {
+        const int k = k0 + 1;
+        c->k = k;
+        int done = 0, st = ST_OK;
+        if (err) {
+          done = 1;
+          st = ST_ERR_TIMEOUT;
+        } else if (!isfinite(e2)) {
+          done = 1;
+          st = ST_ERR_NONFINITE;
+        } else if (e2 <= lim2) {  // ||X - L - S||_F <= tol ||X||_F
+          done = 1;
+        } else if (k >= max_iter) {
+          done = 1;
+          st = ST_NOT_CONVERGED;
+        }
+        if (!done) {
+          const double nxt = schedule == 0 ? fmin(rho * mu_nxt, mu_max) : mu_nxt;
+          c->mu_cur = mu_nxt;
+          c->inv_cur = inv_nxt;
+          c->mu_nxt = nxt;
+          c->f_mu = (float)mu_nxt;
+          c->f_inv_mu = (float)inv_nxt;
+          c->f_gamma = (float)(lambda * inv_nxt);
+          tau = inv_nxt;
+        }
+        c->res2 = e2;
+        c->done = done;
+        c->status = st;
+        stop = done;
+        tail = !done;
+      }
+      if (!stop && (flags & EF_INIT)) {
+        c->normX2 = e2;
+        c->normX = sqrt(e2);
+        c->normX1 = l1;
+        c->lim2 = tol * tol * e2;
+        int done = 0;
+        if (!isfinite(e2)) {
+          done = 1;
+          c->status = ST_ERR_NONFINITE;
+        } else if (e2 == 0.0) {
+          done = 1;
+          c->status = ST_OK;
+        }
+        c->done = done;
+        stop = done;
+        tau = 0.0;
+      }
+      // the timing of the pass that just ran (the first iteration's pass reads
+      // no S, Y and is left out of the steady-state average)
+      if (ts != ~0ull && te > ts) {
+        if (flags & EF_INIT) {
+          c->init_ns = te - ts;
+        } else if ((flags & EF_CHECK) && k0 >= 1) {
+          c->pass_ns += te - ts;
+          c->pass_cnt += 1;
+          if (tl >= ts && t1 >= tl && te >= t1) {
+            c->pass_phase_ns[0] += tl - ts;
+            c->pass_phase_ns[1] += t1 - tl;
+            c->pass_phase_ns[2] += te - t1;
+          }
         }
       }
+      red->t_start = ~0ull;
+      red->t_loop = 0ull;
+      red->t_l1 = 0ull;
+      red->t_end = 0ull;
+      if (stop)
+        set_cond(h, use_cond, 0u);
+      else if (!(flags & EF_EIG))
+        set_cond(h, use_cond, 1u);
+      ec->stop = stop || !(flags & EF_EIG);
+      ec->tail = tail;
+      ec->tau = tau;
     }
-    b.red->t_start = ~0ull;
-    b.red->t_loop = 0ull;
-    b.red->t_l1 = 0ull;
-    b.red->t_end = 0ull;
   }
   __syncthreads();
-  if ((*sFlag)) {
-    if (tid == 0) set_cond(h, use_cond, 0u);
-    return false;
-  }
-  if (flags & EF_CHECK) {
-    if (tid == 0) {
-      const int k = ctrl->k + 1;
-      ctrl->k = k;
-      const double resid = sqrt(b.red->e2) / ctrl->normX;
-      ctrl->resid = resid;
-      int done = 0, st = ST_OK;
-      if (b.red->err) {
-        done = 1;
-        st = ST_ERR_TIMEOUT;
-      } else if (!isfinite(resid)) {
-        done = 1;
-        st = ST_ERR_NONFINITE;
-      } else if (resid <= ctrl->tol) {
-        done = 1;
-      } else if (k >= ctrl->max_iter) {
-        done = 1;
-        st = ST_NOT_CONVERGED;
-      }
-      if (!done) {
-        ctrl->mu_cur = ctrl->mu_nxt;
-        ctrl->mu_nxt = (ctrl->schedule == 0) ? fmin(ctrl->rho * ctrl->mu_cur, ctrl->mu_max) : ctrl->mu_cur;
-        refresh_f32(ctrl);
-      }
-      ctrl->done = done;
-      ctrl->status = st;
-      (*sFlag) = done;
-    }
-    __syncthreads();
-    if ((*sFlag)) {
-      if (tid == 0) set_cond(h, use_cond, 0u);
-      return false;
-    }
-  }
-  if (flags & EF_INIT) {
-    if (tid == 0) {
-      const double x2 = b.red->e2;
-      ctrl->normX2 = x2;
-      ctrl->normX = sqrt(x2);
-      ctrl->normX1 = b.red->l1;
-      int done = 0;
-      if (!isfinite(x2)) {
-        done = 1;
-        ctrl->status = ST_ERR_NONFINITE;
-      } else if (x2 == 0.0) {
-        done = 1;
-        ctrl->status = ST_OK;
-        ctrl->resid = 0.0;
-      }
-      ctrl->done = done;
-      (*sFlag) = done;
-    }
-    __syncthreads();
-    if ((*sFlag)) {
-      if (tid == 0) set_cond(h, use_cond, 0u);
-      return false;
-    }
-  }
-  if (!(flags & EF_EIG)) {
-    if (tid == 0) set_cond(h, use_cond, 1u);
-    return false;
-  }
-  return true;
+  return !ec->stop;
 }
 
-template <int TB, typename Real>
-__global__ void __launch_bounds__(512) eig_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,
-                                                  int use_cond, const double* Gin, double* Vout,
-                                                  double* evals_out) {
+// 1 / mu_nxt after an EF_CHECK step, by one thread, before the step ends.
+static __device__ __forceinline__ void eig_control_tail(Bufs b, const EigCtl* ec) {
+  if (ec->tail) refresh_next(b.ctrl);
+}
+
+// Cyclic Jacobi of an external T x T FP64 matrix (row-major Gin), one CTA: the
+// kernel-level entry rpca_eig.
+template <int TB>
+__global__ void __launch_bounds__(512) eig_kernel(Bufs b, const double* Gin, double* Vout, double* evals_out) {
+  using Real = double;
   constexpr int NP = TB / 2;
   constexpr int LD = TB + 1;
   __shared__ Real sG[2][TB * LD];
@@ -968,38 +993,21 @@ __global__ void __launch_bounds__(512) eig_kernel(Bufs b, int flags, cudaGraphCo
   __shared__ Real sWt[TB][2];
   __shared__ int sI[TB][2];
   __shared__ int sAct[TB];
-  __shared__ double sEv[TB];
-  __shared__ double sGd[TB];
-  __shared__ int sFlag;
-  __shared__ double sTau;
 
-  Ctrl* ctrl = b.ctrl;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int T = b.T;
-  const bool raw = (flags & EF_RAW) != 0;
-  const unsigned long long t0 = gtimer();
-
-  if (!raw && !eig_control(b, flags, h, use_cond, &sFlag)) return;
-
-  // ---- load the Gram and the basis ----
-  const bool cold = raw || (flags & EF_INIT);
   for (int i = tid; i < TB * TB; i += nthr) {
     const int r = i / TB, c = i % TB;
-    const bool in = (r < T && c < T);
-    Real g = 0;
-    if (in) g = Gin ? (Real)Gin[r * T + c] : (Real)b.red->G[r * kMaxT + c];
-    sG[0][r * LD + c] = g;
-    Real v = (r == c) ? (Real)1 : (Real)0;
-    if (!cold && in) v = (Real)b.eig->V32[r * kMaxT + c];
-    sV[0][r * LD + c] = v;
+    sG[0][r * LD + c] = (r < T && c < T) ? Gin[r * T + c] : 0.0;
+    sV[0][r * LD + c] = (r == c) ? 1.0 : 0.0;
   }
   if (tid < TB) sAct[tid] = 0;
   __syncthreads();
 
   // ---- cyclic Jacobi, parallel round-robin ordering ----
   int cur = 0;
-  const Real eps = raw ? (Real)(sizeof(Real) == 8 ? 1e-15 : 1e-7) : (Real)ctrl->jacobi_eps;
-  const int max_sweeps = raw ? 40 : ((cold || (flags & EF_FULL)) ? ctrl->cold_sweeps : ctrl->warm_sweeps);
+  const Real eps = 1e-15;
+  const int max_sweeps = 40;
   int sweeps = 0;
   while (sweeps < max_sweeps) {
     int need = 0;
@@ -1064,74 +1072,11 @@ __global__ void __launch_bounds__(512) eig_kernel(Bufs b, int flags, cudaGraphCo
     }
   }
 
-  if (tid < TB) sEv[tid] = (double)sG[cur][tid * LD + tid];
-  __syncthreads();
-
-  if (raw) {
-    for (int i = tid; i < T * T; i += nthr) {
-      const int r = i / T, c = i % T;
-      Vout[r * T + c] = (double)sV[cur][r * LD + c];
-    }
-    if (tid < T) evals_out[tid] = sEv[tid];
-    if (tid == 0) ctrl->sweeps = sweeps;
-    return;
-  }
-
-  // ---- orthonormality refresh of the basis: V <- V (3I - V^T V)/2 ----
-  {
-    const int nxt = cur ^ 1;
-    // sG[nxt] <- V^T V  (T x T), then sV[nxt] <- V (1.5 I - 0.5 V^T V)
-    for (int i = tid; i < TB * TB; i += nthr) {
-      const int a = i / TB, c = i % TB;
-      Real s = 0;
-      for (int r = 0; r < TB; ++r) s += sV[cur][r * LD + a] * sV[cur][r * LD + c];
-      sG[nxt][a * LD + c] = (a == c ? (Real)1.5 : (Real)0) - (Real)0.5 * s;
-    }
-    __syncthreads();
-    for (int i = tid; i < TB * TB; i += nthr) {
-      const int r = i / TB, c = i % TB;
-      Real s = 0;
-      for (int a = 0; a < TB; ++a) s += sV[cur][r * LD + a] * sG[nxt][a * LD + c];
-      sV[nxt][r * LD + c] = s;
-    }
-    __syncthreads();
-    cur = nxt;
-  }
-
-  // ---- FP64 decisions: mu (first call), tau, sigma > tau, g ----
-  if (tid == 0) {
-    if (flags & EF_INIT) {
-      double lmax = 0.0;
-      for (int a = 0; a < T; ++a) lmax = fmax(lmax, sEv[a]);
-      init_mu(b, lmax);
-    }
-    sTau = 1.0 / ctrl->mu_cur;
-  }
-  __syncthreads();
-  int keep = 0;
-  if (tid < TB) {
-    const double sig = sqrt(fmax(sEv[tid], 0.0));
-    keep = (tid < T) && (sig > sTau);
-    sGd[tid] = keep ? sTau / sig : 1.0;
-  }
-  const int rank = __syncthreads_count(keep);
-
   for (int i = tid; i < T * T; i += nthr) {
-    const int a = i / T, c = i % T;
-    Real s = 0;
-    for (int j = 0; j < T; ++j) s += sV[cur][a * LD + j] * (Real)sGd[j] * sV[cur][c * LD + j];
-    b.eig->Wbar[a * kMaxT + c] = (float)s;
-    b.eig->V32[a * kMaxT + c] = (float)sV[cur][a * LD + c];
+    const int r = i / T, c = i % T;
+    Vout[r * T + c] = sV[cur][r * LD + c];
   }
-  if (tid < T) b.eig->evals[tid] = sEv[tid];
-  if (tid == 0) {
-    ctrl->rank = rank;
-    ctrl->sweeps = sweeps;
-    ctrl->total_sweeps += sweeps;
-    ctrl->eig_ns += gtimer() - t0;
-    ctrl->eig_cnt += 1;
-    set_cond(h, use_cond, 1u);
-  }
+  if (tid < T) evals_out[tid] = sG[cur][tid * LD + tid];
 }
 
 // ---------------------------------------------------------------------------
@@ -1268,7 +1213,7 @@ static __global__ void begin_kernel(Bufs b, const float* X, float* L, float* S, 
     c->rank = 0;
     c->sweeps = 0;
     c->total_sweeps = 0;
-    c->resid = 0.0;
+    c->res2 = 0.0;
     c->pass_ns = c->pass_cnt = c->eig_ns = c->eig_cnt = c->init_ns = 0ull;
     for (int i = 0; i < 4; ++i) c->eig_phase_ns[i] = 0ull;
     for (int i = 0; i < 3; ++i) c->pass_phase_ns[i] = 0ull;
@@ -1284,7 +1229,7 @@ static __global__ void begin_kernel(Bufs b, const float* X, float* L, float* S, 
 #include "rpca_tc.cuh"
 #include "rpca_pass_tc.cuh"
 #include "rpca_pass_fs.cuh"
-#include "rpca_eig_fast.cuh"
+#include "rpca_jacobi.cuh"
 #include "rpca_eig64.cuh"
 
 }  // namespace rpca

@@ -32,6 +32,7 @@ WideKernels make_wide() {
   k.pass_threads = kWideThreads;
   k.eig = (void*)eig_wide_kernel;
   k.eig_threads = kEigWThreads;
+  k.eig_ctas = kEigWRanks;
   for (int i = 0; i < 4; ++i) {
     k.pass_tc[i] = nullptr;
     k.pass_tc_smem[i] = 0;
@@ -48,6 +49,8 @@ WideKernels make_wide() {
   }
   return k;
 }
+
+size_t wide_eig_scr_bytes(int T) { return eig_scr_bytes(T); }
 
 size_t wide_tc_img_bytes(int T, int precision) {
   const int TP = wtc_tp(T);
@@ -82,7 +85,10 @@ bool wide_kernels(int T, bool cplx, bool force, WideKernels* out) {
   if (cplx && (T & 1)) return false;
   const int TP = (T + 31) / 32 * 32;
   *out = cplx ? pick_wide<true>(TP) : pick_wide<false>(TP);
-  out->eig_smem = eig_wide_smem(T, kVRows);
+  // the sweeps' columns, or one rank's operands of a product, as far as they fit
+  const size_t ops = 2 * sizeof(float) * (size_t)T * (eig_ld(T) + (eig_ld(T) / 4 + kEigWRanks - 1) / kEigWRanks * 4);
+  out->eig_smem = eig_wide_smem(T);
+  if (ops > out->eig_smem) out->eig_smem = ops < kEigWMaxSmem ? ops : (out->eig_smem > kEigWMaxSmem ? out->eig_smem : kEigWMaxSmem);
   if (cudaFuncSetAttribute(out->eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out->eig_smem) != cudaSuccess)
     return false;
   for (int i = 0; i < 4; ++i)

@@ -18,14 +18,7 @@
 //      (4 x 4 blocks of the upper triangle spread over the CTA's threads).
 // The CTA partials go through the same two-level reduction as the narrow path.
 //
-// The eigen-step (one CTA of 1024 threads) runs cyclic Jacobi with FP32
-// rotations on the rotated Gram held in shared memory: each round of the
-// round-robin order rotates T/2 disjoint pairs; every 2 x 2 block of pairs is
-// then updated in place by one thread (the four entries of a block depend
-// only on each other), and the rotations are applied to the columns of V
-// (kept in the workspace) in the same phase.  The decisions (sigma, tau, the
-// rank and the first mu) are FP64, and Wbar = V diag(g) V^T is formed with V
-// staged in shared memory.
+// The eigen-step is in rpca_eig_wide.cuh.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -42,20 +35,6 @@ constexpr int kWP = 32;           // pixels per tile (one per lane)
 constexpr int kResLd = 4;
 constexpr int kWKC = 32;          // rows of Wbar / V staged per step
 constexpr int kWideThreads = 256;
-constexpr int kEigWThreads = 1024;
-constexpr int kVRows = 16;        // rows of V staged per step of V <- V + V D (stand-alone kernel)
-
-// Upper-triangle block (A, C), A <= C < K, of linear index idx in row order
-// (row A holds K - A blocks): closed form with one correction step.
-__device__ __forceinline__ void tri_coords(int idx, int K, int& A, int& C) {
-  const float k2 = 2.f * K + 1.f;
-  int a = (int)floorf(0.5f * (k2 - sqrtf(fmaxf(k2 * k2 - 8.f * (float)idx, 0.f))));
-  a = max(0, min(a, K - 1));
-  while (a > 0 && a * K - a * (a - 1) / 2 > idx) --a;
-  while (a + 1 < K && (a + 1) * K - (a + 1) * a / 2 <= idx) ++a;
-  A = a;
-  C = a + (idx - (a * K - a * (a - 1) / 2));
-}
 
 template <int CW>
 struct WideShape {
@@ -787,479 +766,6 @@ __device__ __forceinline__ void wtc_images(const Bufs& b) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Eigen-step for wide windows (one CTA; the stand-alone kernel uses kEigWThreads threads).
-// ---------------------------------------------------------------------------
-// Windows up to this many frames keep D = Q - I (the product of the step's
-// rotations, minus I) in shared memory beside G and update it in every round
-// (each round's items are independent, so the CTA shares them); larger ones
-// log the rotations and replay them onto D after the sweeps, when G is
-// consumed.
-constexpr int kWideInlineDMaxT = 144;
-__host__ __device__ constexpr bool eig_wide_inline_d(int T) { return T <= kWideInlineDMaxT; }
-
-// The eigen-step on one CTA of any multiple of 32 threads; `eigw_smem` holds
-// eig_wide_smem(T, vrows) bytes.
-__host__ __device__ constexpr size_t eig_wide_smem(int T, int vrows) {
-  return sizeof(float) * ((size_t)(eig_wide_inline_d(T) ? 2 : 1) * (T + (T & 1)) * (T + (T & 1) + 1) +
-                          (size_t)vrows * T);
-}
-
-static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond, float* eigw_smem,
-                              int vrows) {
-  __shared__ float sC[kMaxTW / 2], sSn[kMaxTW / 2];
-  __shared__ float sDp[kMaxTW / 2], sDq[kMaxTW / 2];
-  __shared__ float sCm1[kMaxTW / 2];  // c - 1 = -s^2 / (1 + c) of every pair slot of the round
-  __shared__ double sEv[kMaxTW];
-  __shared__ float sG[kMaxTW];
-  __shared__ int sAct[kMaxTW / 2], sPos[kMaxTW / 2];
-  __shared__ int4 sPair[kMaxTW / 2];    // (p, q, c, s) of every pair slot of the round
-  __shared__ int sWarpCnt[(kMaxTW / 2 + 31) / 32];
-  __shared__ int sFlag;
-  __shared__ double sTau;
-
-  Ctrl* ctrl = b.ctrl;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int T = b.T;
-  const int Te = T + (T & 1);   // even size (a zero row/column pads odd T)
-  const int K = Te / 2;
-  const int LD = Te + 1;
-  float* G = eigw_smem;          // [Te][LD]
-  const bool inline_d = eig_wide_inline_d(T);
-  float* Dn = eigw_smem + (size_t)Te * LD;  // [Te][LD]: D = Q - I, updated per round (inline_d)
-  float* after = eigw_smem + (size_t)(inline_d ? 2 : 1) * Te * LD;  // staging beyond G (and D)
-  const unsigned long long t0 = gtimer();
-  if (!eig_control(b, flags, h, use_cond, &sFlag)) return;
-  const bool cold = (flags & EF_INIT) != 0;
-
-  for (int i = tid; i < Te * LD; i += nthr) {
-    const int r = i / LD, c = i % LD;
-    G[i] = (r < T && c < T) ? b.Gw[r * T + c] : 0.f;
-  }
-  if (cold)
-    for (int i = tid; i < T * T; i += nthr) b.Vw[i] = (i / T == i % T) ? 1.f : 0.f;
-  if (inline_d)
-    for (int i = tid; i < Te * LD; i += nthr) Dn[i] = 0.f;
-  __syncthreads();  // (global writes of the block are visible to its later reads)
-  const unsigned long long t1 = gtimer();
-
-  const float eps = (float)ctrl->jacobi_eps;
-  const float eps2 = eps * eps;
-  int max_sweeps = (cold || (flags & EF_FULL)) ? ctrl->cold_sweeps : ctrl->warm_sweeps;
-  if (max_sweeps > kWideLogSweeps) max_sweeps = kWideLogSweeps;
-  int sweeps = 0, rounds_run = 0;
-  // Each round's rotated pairs are logged (round number, count, slots and
-  // (c, s)) to the workspace and applied to V after the sweeps, with V staged
-  // in shared memory.
-  float2* log_cs = b.rot_log;   // (c, s) of every rotated pair, round after round
-  int* log_k = b.rot_k;          // its columns p | q << 8, bit 16 on the first rotation of a round
-  int* log_rnd = b.rot_rnd;      // per logged round: round number, rotated pairs
-  const int KW = (K + 31) / 32;  // warps covering the pair slots
-  int logged = 0;                // entries logged so far
-  while (sweeps < max_sweeps) {
-    int need = 0;
-    for (int i = tid; i < Te * Te; i += nthr) {
-      const int a = i / Te, c = i % Te;
-      if (a < c) {
-        const float apq = G[a * LD + c];
-        if (apq != 0.f && apq * apq > eps2 * fabsf(G[a * LD + a] * G[c * LD + c])) need = 1;
-      }
-    }
-    if (!__syncthreads_or(need)) break;
-    for (int rnd = 0; rnd < Te - 1; ++rnd) {
-      // ---- phase A: the round's rotations (GVL sym.schur2, FP32) ----
-      int act = 0;
-      if (tid < K) {
-        int pa, pb;
-        rr_pair(rnd, tid, Te, pa, pb);
-        const int p = min(pa, pb), q = max(pa, pb);
-        const float app = G[p * LD + p], aqq = G[q * LD + q], apq = G[p * LD + q];
-        float c = 1.f, s = 0.f, dp = app, dq = aqq;
-        if (apq != 0.f && apq * apq > eps2 * fabsf(app * aqq)) {
-          act = 1;
-          const float dd = aqq - app;
-          const float r2 = fmaf(dd, dd, 4.f * apq * apq);
-          const float den = fabsf(dd) + sqrtf(r2);
-          const float t = copysignf(1.f, dd) * (2.f * apq) * __fdividef(1.f, den);
-          c = rsqrtf(fmaf(t, t, 1.f));
-          s = t * c;
-          dp = app - t * apq;
-          dq = aqq + t * apq;
-        }
-        sC[tid] = c;
-        sSn[tid] = s;
-        sCm1[tid] = -s * s / (1.f + c);
-        sDp[tid] = dp;
-        sDq[tid] = dq;
-        sPair[tid] = make_int4(p, q, __float_as_int(c), __float_as_int(s));
-      }
-      // compact list of the rotated pairs (ballot per warp, then prefix)
-      unsigned bal = 0u;
-      if (tid < 32 * KW) {
-        bal = __ballot_sync(0xffffffffu, act);
-        if ((tid & 31) == 0) sWarpCnt[tid >> 5] = __popc(bal);
-      }
-      __syncthreads();
-      int na = 0, off = 0;
-      for (int wq = 0; wq < KW; ++wq) {
-        if (wq < (tid >> 5)) off += sWarpCnt[wq];
-        na += sWarpCnt[wq];
-      }
-      if (na == 0) {  // (uniform: every thread read the same counts)
-        __syncthreads();  // the counts are read before the next round rewrites them
-        continue;
-      }
-      if (tid < K) {
-        // (each slot has one writer, and the previous round's readers passed
-        // its closing barrier)
-        int pos = -1;
-        if (act) {
-          pos = off + __popc(bal & ((1u << (tid & 31)) - 1u));
-          sAct[pos] = tid;
-          if (!inline_d) {
-            // the replay needs the pair's columns and where each round starts
-            const int4 pr = sPair[tid];
-            log_k[logged + pos] = pr.x | (pr.y << 8) | (pos == 0 ? (1 << 16) : 0);
-            log_cs[logged + pos] = make_float2(sC[tid], sSn[tid]);
-          }
-        }
-        sPos[tid] = pos;
-      }
-      if (tid == 0 && !inline_d) {
-        log_rnd[2 * rounds_run] = rnd;
-        log_rnd[2 * rounds_run + 1] = na;
-      }
-      logged += na;
-      ++rounds_run;
-      __syncthreads();
-      // ---- phase B: G <- J^T G J on every 2 x 2 block of pairs that holds a
-      //      rotated pair (a block of two rotated pairs once), in place ----
-      // warp w takes rotated pairs w, w + 32, ...; lane l takes partner pairs
-      // l, l + 32, ... (the rotated pair's values are read once per warp row;
-      // a partner's (p, q, c, s) is one 16-byte load)
-      for (int ai = tid >> 5; ai < na; ai += nthr / 32) {
-        const int A = sAct[ai];
-        const int4 pa4 = sPair[A];
-        const int pA = pa4.x, qA = pa4.y;
-        const float cA = __int_as_float(pa4.z), sA = __int_as_float(pa4.w);
-        for (int C = tid & 31; C < K; C += 32) {
-        if (C == A) {
-          G[pA * LD + pA] = sDp[A];
-          G[qA * LD + qA] = sDq[A];
-          G[pA * LD + qA] = 0.f;
-          G[qA * LD + pA] = 0.f;
-          continue;
-        }
-        const int pc = sPos[C];
-        if (pc >= 0 && pc < ai) continue;  // the block of two rotated pairs belongs to the earlier one
-        const int4 pc4 = sPair[C];
-        const int pC = pc4.x, qC = pc4.y;
-        const float cC = __int_as_float(pc4.z), sC_ = __int_as_float(pc4.w);
-        const float g00 = G[pA * LD + pC], g01 = G[pA * LD + qC];
-        const float g10 = G[qA * LD + pC], g11 = G[qA * LD + qC];
-        // columns of J for the pair: p -> (c, -s), q -> (s, c)
-        const float h00 = cC * g00 - sC_ * g01, h01 = sC_ * g00 + cC * g01;  // G J (rows pA)
-        const float h10 = cC * g10 - sC_ * g11, h11 = sC_ * g10 + cC * g11;  // G J (rows qA)
-        const float n00 = cA * h00 - sA * h10, n01 = cA * h01 - sA * h11;    // J^T (G J)
-        const float n10 = sA * h00 + cA * h10, n11 = sA * h01 + cA * h11;
-        G[pA * LD + pC] = n00;
-        G[pC * LD + pA] = n00;
-        G[pA * LD + qC] = n01;
-        G[qC * LD + pA] = n01;
-        G[qA * LD + pC] = n10;
-        G[pC * LD + qA] = n10;
-        G[qA * LD + qC] = n11;
-        G[qC * LD + qA] = n11;
-        }
-      }
-      if (inline_d) {
-        // D' = D J + (J - I) on the round's rotated pairs: (row r, rotated
-        // pair) touches D[r][p] and D[r][q] only; lane = rotated pair, warp =
-        // rows
-        const int warp = tid >> 5, lane = tid & 31, nwarps = nthr >> 5;
-        for (int ai = lane; ai < na; ai += 32) {
-          const int A = sAct[ai];
-          const int4 pr = sPair[A];
-          const int p = pr.x, q = pr.y;
-          const float c = __int_as_float(pr.z), sn = __int_as_float(pr.w), cm1 = sCm1[A];
-          for (int r = warp; r < T; r += nwarps) {
-            float* dr = &Dn[r * LD];
-            const float dp = dr[p], dq = dr[q];
-            float np = fmaf(c, dp, -sn * dq), nq = fmaf(sn, dp, c * dq);
-            if (r == p) {
-              np += cm1;
-              nq += sn;
-            } else if (r == q) {
-              np -= sn;
-              nq += cm1;
-            }
-            dr[p] = np;
-            dr[q] = nq;
-          }
-        }
-      }
-      __syncthreads();
-    }
-    ++sweeps;
-  }
-  const unsigned long long t2 = gtimer();
-  if (tid < T) sEv[tid] = (double)G[tid * LD + tid];
-  __syncthreads();
-
-  // ---- Q = J_1 J_2 ... kept as D = Q - I: near the identity D is small, so
-  //      its rounding errors are relative to small entries; then V <- V + V D.
-  //      Inline: D is already complete; else replay the logged rounds onto D
-  //      over the consumed G ----
-  float* D = inline_d ? Dn : G;  // [T][LD]
-  if (!inline_d)
-    for (int i = tid; i < T * LD; i += nthr) D[i] = 0.f;
-  // The rows of D are independent (D' = D J + (J - I) mixes columns p and q
-  // of each row) and warp w owns rows w, w + nwarps, ..., so between rounds
-  // only a warp has to wait for itself.  The CTA stages the log a chunk at a
-  // time into shared memory (over the V staging rows, free until the update
-  // below; one barrier per chunk); each warp walks the chunk 32 entries at a
-  // time, lane = rotation, and applies the rotations of one round (a run of
-  // entries starting at a flagged one) before those of the next.
-  if (!inline_d) {
-    const int nwarps = nthr >> 5, warp = tid >> 5, lane = tid & 31;
-    float2* stc = reinterpret_cast<float2*>(after);
-    const int E = max(1, (vrows * T * (int)sizeof(float)) / (int)(sizeof(float2) + sizeof(int)));
-    int* stp = reinterpret_cast<int*>(stc + E);
-    for (int c0 = 0; c0 < logged; c0 += E) {
-      const int ne = min(E, logged - c0);
-      __syncthreads();  // (D zeroed; the previous chunk consumed)
-      for (int i = tid; i < ne; i += nthr) {
-        stc[i] = __ldcg(&log_cs[c0 + i]);
-        stp[i] = __ldcg(&log_k[c0 + i]);
-      }
-      __syncthreads();
-      for (int w0 = 0; w0 < ne; w0 += 32) {
-        const int i = w0 + lane;
-        const bool have = i < ne;
-        const int pk = have ? stp[i] : 0;
-        const float2 cs = have ? stc[i] : make_float2(1.f, 0.f);
-        const unsigned starts = __ballot_sync(0xffffffffu, have && (pk >> 16) != 0);
-        const int p = pk & 255, q = (pk >> 8) & 255;
-        // Q' = Q J  <=>  D' = D J + (J - I); c - 1 = -s^2 / (1 + c)
-        const float c = cs.x, sn = cs.y, cm1 = -sn * sn / (1.f + c);
-        const int nlive = min(32, ne - w0);
-        for (int lo = 0; lo < nlive;) {
-          const unsigned later = lo < 31 ? (starts & ~((2u << lo) - 1u)) : 0u;
-          const int hi = later ? __ffs(later) - 1 : 32;
-          if (lane >= lo && lane < hi && have && q < T) {
-            for (int r = warp; r < T; r += nwarps) {
-              float* dr = &D[r * LD];
-              const float dp = dr[p], dq = dr[q];
-              float np = fmaf(c, dp, -sn * dq), nq = fmaf(sn, dp, c * dq);
-              if (r == p) {
-                np += cm1;
-                nq += sn;
-              } else if (r == q) {
-                np -= sn;
-                nq += cm1;
-              }
-              dr[p] = np;
-              dr[q] = nq;
-            }
-          }
-          __syncwarp();
-          lo = hi;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  // V <- V + V D, vrows rows of V at a time staged after D
-  float* sVo = after;  // [vrows][T]
-  for (int r0 = 0; r0 < T; r0 += vrows) {
-    const int nr = min(vrows, T - r0);
-    for (int i = tid; i < nr * T; i += nthr) sVo[i] = __ldcg(&b.Vw[(size_t)r0 * T + i]);
-    __syncthreads();
-    const int ncg = (T + 3) / 4;
-    for (int item = tid; item < nr * ncg; item += nthr) {
-      const int rr = item / ncg, c0 = 4 * (item % ncg);
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      int cc[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) cc[k] = min(c0 + k, T - 1);
-      for (int j = 0; j < T; ++j) {
-        const float v = sVo[rr * T + j];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = fmaf(v, D[j * LD + cc[k]], acc[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (c0 + k < T) b.Vw[(size_t)(r0 + rr) * T + c0 + k] = sVo[rr * T + c0 + k] + acc[k];
-    }
-    __syncthreads();
-  }
-  // V (new) staged over D for the orthonormalisation and Wbar
-  float* sV = G;  // [T][T + 1]
-  const int LV = T + 1;
-  for (int i = tid; i < T * T; i += nthr) sV[(i / T) * LV + i % T] = __ldcg(&b.Vw[i]);
-  __syncthreads();
-
-  // ---- FP64 decisions ----
-  if (tid == 0) {
-    if (flags & EF_INIT) {
-      double lmax = 0.0;
-      for (int a = 0; a < T; ++a) lmax = fmax(lmax, sEv[a]);
-      init_mu(b, lmax);
-    }
-    sTau = 1.0 / ctrl->mu_cur;
-  }
-  __syncthreads();
-  int keep = 0;
-  if (tid < T) {
-    const double sig = sqrt(fmax(sEv[tid], 0.0));
-    keep = sig > sTau;
-    sG[tid] = keep ? (float)(sTau / sig) : 1.f;
-  }
-  const int rank = __syncthreads_count(keep);
-  // ---- re-orthonormalise V (one Newton-Schulz step, V <- V (3 I - V^T V) / 2),
-  //      then Wbar = V diag(g) V^T; V is staged over G ----
-  const int NB4 = (T + 3) / 4;
-  const int nb2 = NB4 * (NB4 + 1) / 2;
-  const unsigned long long t3 = gtimer();
-  // A = V^T V into the (consumed) Gram array, and its largest deviation from I
-  float dev = 0.f;
-  for (int bidx = tid; bidx < nb2; bidx += nthr) {
-    int bi, bj;
-    blk_coords(bidx, NB4, bi, bj);
-    float acc[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-    int ca[4], cc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      ca[i] = min(4 * bi + i, T - 1);
-      cc[i] = min(4 * bj + i, T - 1);
-    }
-    for (int r = 0; r < T; ++r) {
-      float va[4], vc[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        va[i] = sV[r * LV + ca[i]];
-        vc[i] = sV[r * LV + cc[i]];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[i * 4 + k] = fmaf(va[i], vc[k], acc[i * 4 + k]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int a = 4 * bi + i, c = 4 * bj + k;
-        if (a < T && c < T) {
-          b.Gw[a * T + c] = acc[i * 4 + k];
-          b.Gw[c * T + a] = acc[i * 4 + k];
-          dev = fmaxf(dev, fabsf(acc[i * 4 + k] - (a == c ? 1.f : 0.f)));
-        }
-      }
-  }
-  // skip the correction once V is orthonormal to FP32 rounding
-  const int correct = __syncthreads_or(dev > 4e-7f);
-  if (correct) {
-    // V_new = 1.5 V - 0.5 V A  (rows of V from shared memory, A from the workspace)
-    const int nbf = NB4 * NB4;
-    for (int bidx = tid; bidx < nbf; bidx += nthr) {
-      const int bi = bidx / NB4, bj = bidx % NB4;
-      float acc[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-      int ra[4], cc[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ra[i] = min(4 * bi + i, T - 1);
-        cc[i] = min(4 * bj + i, T - 1);
-      }
-      for (int j = 0; j < T; ++j) {
-        float va[4], ac[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          va[i] = sV[ra[i] * LV + j];
-          ac[i] = __ldcg(&b.Gw[j * T + cc[i]]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) acc[i * 4 + k] = fmaf(va[i], ac[k], acc[i * 4 + k]);
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int r = 4 * bi + i, c = 4 * bj + k;
-          if (r < T && c < T) b.Vw[r * T + c] = 1.5f * sV[r * LV + c] - 0.5f * acc[i * 4 + k];
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < T * T; i += nthr) sV[(i / T) * LV + i % T] = __ldcg(&b.Vw[i]);
-    __syncthreads();
-  }
-  for (int bidx = tid; bidx < nb2; bidx += nthr) {
-    int bi, bj;
-    blk_coords(bidx, NB4, bi, bj);
-    float acc[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-    int ra[4], rc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      ra[i] = min(4 * bi + i, T - 1);
-      rc[i] = min(4 * bj + i, T - 1);
-    }
-    for (int j = 0; j < T; ++j) {
-      const float gj = sG[j];
-      float va[4], vc[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        va[i] = sV[ra[i] * LV + j] * gj;
-        vc[i] = sV[rc[i] * LV + j];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[i * 4 + k] = fmaf(va[i], vc[k], acc[i * 4 + k]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int a = 4 * bi + i, c = 4 * bj + k;
-        if (a < T && c < T) {
-          b.Ww[a * T + c] = acc[i * 4 + k];
-          b.Ww[c * T + a] = acc[i * 4 + k];
-        }
-      }
-  }
-  if (b.wtc) {
-    __syncthreads();  // Ww written by the whole CTA
-    wtc_images(b);
-  }
-  if (tid < T) b.evw[tid] = sEv[tid];
-  if (tid == 0) {
-    ctrl->rank = rank;
-    ctrl->sweeps = sweeps;
-    ctrl->total_sweeps += sweeps;
-    const unsigned long long t4 = gtimer();
-    ctrl->eig_ns += t4 - t0;
-    ctrl->eig_cnt += 1;
-    ctrl->eig_phase_ns[0] += t1 - t0;
-    ctrl->eig_phase_ns[1] += t2 - t1;
-    ctrl->eig_phase_ns[2] += t3 - t2;
-    ctrl->eig_phase_ns[3] += t4 - t3;
-    ctrl->eig_rounds += rounds_run;
-    set_cond(h, use_cond, 1u);
-  }
-}
-
-static __global__ void __launch_bounds__(kEigWThreads, 1) eig_wide_kernel(Bufs b, int flags,
-                                                                          cudaGraphConditionalHandle h, int use_cond) {
-  extern __shared__ __align__(16) float eigw_smem[];
-  eig_wide_body(b, flags, h, use_cond, eigw_smem, kVRows);
-}
+#include "rpca_eig_wide.cuh"
 
 }  // namespace rpca
