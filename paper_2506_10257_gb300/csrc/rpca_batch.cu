@@ -68,8 +68,8 @@ struct KernelInfo {
   size_t smem;
 };
 
-// Columns per warp of the tiled pass for T real columns.
-int wide_cw(int Tr) { return (Tr + 31) / 32 * 32 / 8; }
+// Pixels per tile of the tiled pass in a batch (its lanes are far fewer CTAs than a plan's grid).
+int wide_rp(int Tr, bool cplx) { return tile_tp(Tr, cplx) > 128 ? 64 : 128; }
 
 KernelInfo batch_kernel_for(int tbmax) {
   if (tbmax <= 20) return {(void*)batch_kernel<20>, batch_smem<20>()};
@@ -91,6 +91,7 @@ struct rpca_batch_s {
   std::vector<PlanView> views;
   KernelInfo kern{};
   bool wide = false;           // every window runs the tiled bodies
+  int threads() const { return wide ? kWideThreads : kBatchThreads; }
   int sms = 0;
   int occ_max = 0;       // resident batch CTAs per SM the kernel allows
   BatchConfig cfg{};
@@ -226,7 +227,8 @@ void make_schedule(rpca_batch_s* b, const BatchConfig& cfg) {
     for (int w : lw[l]) {
       b->win_slot[w] = (int)b->slot_win.size();
       b->slot_win.push_back(w);
-      const int64_t tiles = (b->p[w].m + b->views[w].tile - 1) / b->views[w].tile;
+      const int tile = b->wide ? wide_rp(b->views[w].T, b->views[w].cplx) : b->views[w].tile;
+      const int64_t tiles = (b->p[w].m + tile - 1) / tile;
       b->win_ncta[w] =
           (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)pass_ctas, tiles, b->views[w].max_grid}));
     }
@@ -248,7 +250,7 @@ cudaError_t launch_batch(rpca_batch_s* b, cudaStream_t s) {
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
   lc.gridDim = dim3((unsigned)b->grid);
-  lc.blockDim = dim3(kBatchThreads);
+  lc.blockDim = dim3(b->threads());
   lc.dynamicSmemBytes = b->kern.smem;
   lc.stream = s;
   cudaLaunchAttribute attr[1];
@@ -316,8 +318,9 @@ void write_static_desc(rpca_batch_s* b) {
     wd.b = b->views[w].bufs;
     wd.b.finalize = 1;
     wd.b.grid = b->win_ncta[w];
+    wd.b.group = kGroup;
     wd.b.ngroups = (b->win_ncta[w] + kGroup - 1) / kGroup;
-    wd.TB = b->wide ? wide_cw(b->views[w].T) : bucket_tb(b->p[w].T);
+    wd.TB = b->wide ? tile_tp(b->views[w].T, b->views[w].cplx) : bucket_tb(b->p[w].T);
   }
 }
 
@@ -417,7 +420,7 @@ rpca_status rpca_batch_create(const rpca_params* params, int32_t n, rpca_batch_t
     size_t need = 0;
     for (int i = 0; i < n; ++i) {
       const int Tr = params[i].dtype == RPCA_C64 ? 2 * params[i].T : params[i].T;
-      need = std::max({need, wide_pass_smem_bytes(wide_cw(Tr)), eig_wide_smem(Tr)});
+      need = std::max({need, tile_pass_smem(Tr, wide_rp(Tr, cplx), cplx), eig_wide_smem(Tr)});
     }
     if (need > room) {
       delete b;
@@ -427,7 +430,7 @@ rpca_status rpca_batch_create(const rpca_params* params, int32_t n, rpca_batch_t
   }
   e = cudaFuncSetAttribute(b->kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->kern.smem);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ_max, b->kern.fn, kBatchThreads, b->kern.smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->occ_max, b->kern.fn, b->threads(), b->kern.smem);
   if (e != cudaSuccess || b->occ_max < 1) {
     delete b;
     return e != cudaSuccess ? cuda_st(e) : RPCA_ERR_UNSUPPORTED;

@@ -15,39 +15,39 @@ namespace rpca {
 
 // The tiled bodies are called, not inlined, into the one kernel that serves
 // every column count: each compiles once, which keeps the build short.
-template <int CW, int MODE, bool CPLX>
+template <int TP, int RP, int MODE, bool CPLX>
 __device__ __noinline__ bool wide_pass_call(Bufs b, int lc, int nc, float* f) {
-  return pass_wide_body<CW, MODE, CPLX>(b, lc, nc, f);
+  return pass_tile_body<TP, RP, MODE, CPLX>(b, lc, nc, f);
 }
 __device__ __noinline__ void wide_eig_call(Bufs b, int flags, float* f, int eig_floats) {
   eig_wide_body<8>(b, flags, 0, 0, f, eig_floats, 0, 1);
 }
 
-template <int CW, bool CPLX>
-struct WideBody {
-  static __device__ bool pass(Bufs b, bool init, int lc, int nc, unsigned char* dsm) {
-    float* f = reinterpret_cast<float*>(dsm);
-    return init ? wide_pass_call<CW, PM_INIT, CPLX>(b, lc, nc, f) : wide_pass_call<CW, PM_FUSED, CPLX>(b, lc, nc, f);
-  }
-  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int eig_floats) {
-    wide_eig_call(b, flags, reinterpret_cast<float*>(dsm), eig_floats);
-  }
-};
-
-// The tiled steps of a window by its columns per warp (TB of the descriptor).
+// The tiled steps of a window by its padded columns (TB of the descriptor).
 template <bool CPLX>
 struct WideDisp {
+  template <int TP>
+  static __device__ bool run(Bufs b, bool init, int lc, int nc, float* f) {
+    constexpr int RP = TP > 128 ? 64 : 128;
+    return init ? wide_pass_call<TP, RP, PM_INIT, CPLX>(b, lc, nc, f) : wide_pass_call<TP, RP, PM_FUSED, CPLX>(b, lc, nc, f);
+  }
   static __device__ bool pass(WinDesc& wd, bool init, int lc, int nc, unsigned char* dsm) {
+    float* f = reinterpret_cast<float*>(dsm);
     switch (wd.TB) {
-      case 4: return WideBody<4, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 8: return WideBody<8, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 12: return WideBody<12, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 16: return WideBody<16, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 20: return WideBody<20, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 24: return WideBody<24, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      case 28: return WideBody<28, CPLX>::pass(wd.b, init, lc, nc, dsm);
-      default: return false;
+      case 32: return run<32>(wd.b, init, lc, nc, f);
+      case 64: return run<64>(wd.b, init, lc, nc, f);
+      case 96: return run<96>(wd.b, init, lc, nc, f);
+      case 128: return run<128>(wd.b, init, lc, nc, f);
+      case 192: return run<192>(wd.b, init, lc, nc, f);
+      default: break;
     }
+    if constexpr (CPLX) {
+      if (wd.TB == 256) return run<256>(wd.b, init, lc, nc, f);
+    } else {
+      if (wd.TB == 160) return run<160>(wd.b, init, lc, nc, f);
+      if (wd.TB == 224) return run<224>(wd.b, init, lc, nc, f);
+    }
+    return false;
   }
   static __device__ void eig(WinDesc& wd, int flags, unsigned char* dsm, int eig_floats) {
     wide_eig_call(wd.b, flags, reinterpret_cast<float*>(dsm), eig_floats);
@@ -55,9 +55,9 @@ struct WideDisp {
 };
 
 // Batches holding a wide or complex window: every window runs the tiled
-// bodies (TB of a window = its columns per warp, CW).
+// bodies (TB of a window: its padded columns), 16 warps a CTA.
 template <bool CPLX>
-__global__ void __launch_bounds__(kBatchThreads, 1) batch_kernel_wide(BatchDesc* bd) {
+__global__ void __launch_bounds__(kWideThreads, 1) batch_kernel_wide(BatchDesc* bd) {
   extern __shared__ __align__(16) unsigned char batch_dsm[];
   const int nl = bd->nlanes;
   int l = 0;

@@ -100,7 +100,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 struct Layout {
   size_t ctrl, eig, red, job, gw, ww, vw, evw, escr, wtc, gram_part, group_part, scal_part, gscal_part, ybuf,
       total;
-  int grid, ngroups;
+  int grid, ngroups, group;
   int ws_grid;     // CTAs of the passes with 128-pixel tiles (TMA-fed FP32, tiled tensor-core): one per SM
   int wide_grid;   // CTAs of the wide pass (T > kMaxT; one per SM, 32-pixel tiles)
 };
@@ -114,18 +114,21 @@ int device_sms() {
 
 // Grid: one 256-thread CTA per SM (register bound), never more than the tiles.
 // wtc_bytes: B operand images of the tiled tensor-core pass (0: none).
-Layout make_layout(int64_t m, int T, int sms, bool wide, size_t wtc_bytes = 0) {
+Layout make_layout(int64_t m, int T, int sms, bool wide, bool cplx = false, size_t wtc_bytes = 0) {
   Layout L;
   const int64_t ntiles = (m + kTile - 1) / kTile;
   int64_t grid = std::min<int64_t>(ntiles, (int64_t)std::max(sms, 1) * kPassCtasPerSm);
   grid = std::min<int64_t>(grid, (int64_t)kGroup * kMaxGroups);
   L.grid = (int)std::max<int64_t>(grid, 1);
   L.ws_grid = (int)std::max<int64_t>(std::min<int64_t>((m + 127) / 128, std::max(sms, 1)), 1);
-  int wtile = 32, wper = 1;
-  if (wide) wide_launch_shape(T, &wtile, &wper);
+  int wtile = 64, wper = 1;
+  if (wide) wide_launch_shape(T, cplx, m, sms, &wtile, &wper);
   L.wide_grid = (int)std::max<int64_t>(std::min<int64_t>((m + wtile - 1) / wtile, (int64_t)std::max(sms, 1) * wper), 1);
   const int maxgrid = std::max({L.grid, L.ws_grid, wide ? L.wide_grid : 1});
-  L.ngroups = (maxgrid + kGroup - 1) / kGroup;
+  // wide windows: small groups, whose sums of T x T partials are what the pass waits for at its end
+  // (groups of 16 took 39 us of a 760 us pass at 132 frames)
+  L.group = !wide ? kGroup : maxgrid <= 4 * kMaxGroups ? 4 : (maxgrid + kMaxGroups - 1) / kMaxGroups;
+  L.ngroups = (maxgrid + L.group - 1) / L.group;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     size_t o = off;
@@ -440,7 +443,7 @@ rpca_status rpca_workspace_size(const rpca_params* p, size_t* bytes) {
   if (!bytes) return RPCA_ERR_ARG;
   const int sms = device_sms();
   if (sms <= 0) return RPCA_ERR_CUDA;
-  *bytes = make_layout(p->m, real_cols(p), sms, uses_wide(p),
+  *bytes = make_layout(p->m, real_cols(p), sms, uses_wide(p), p->dtype == RPCA_C64,
                        uses_wide(p) ? wide_tc_img_bytes(real_cols(p), p->precision) : 0).total;
   return RPCA_OK;
 }
@@ -472,7 +475,7 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   const int Tr = real_cols(p);
   pl->wide = uses_wide(p) || force_wide;
   if (pl->wide) {
-    if (!wide_kernels(Tr, cplx, pl->wide && !uses_wide(p), &pl->wk)) {
+    if (!wide_kernels(Tr, cplx, pl->wide && !uses_wide(p), p->m, sms, &pl->wk)) {
       delete pl;
       return RPCA_ERR_UNSUPPORTED;
     }
@@ -520,7 +523,7 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
       return cuda_status(ea);
     }
   }
-  pl->lay = make_layout(p->m, Tr, sms, pl->wide, pl->wide ? wide_tc_img_bytes(Tr, p->precision) : 0);
+  pl->lay = make_layout(p->m, Tr, sms, pl->wide, cplx, pl->wide ? wide_tc_img_bytes(Tr, p->precision) : 0);
   if (!pl->wide) {
     cudaError_t ea = cudaFuncSetAttribute(pl->ks.eig_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)pl->ks.eig_step_smem);
@@ -566,6 +569,7 @@ static rpca_status plan_create_impl(const rpca_params* p, void* workspace, size_
   b.wide = pl->wide ? 1 : 0;
   b.grid = pl->lay.grid;
   b.ngroups = pl->lay.ngroups;
+  b.group = pl->lay.group;
   // a sharded plan's passes finish their reduction themselves, so the summed
   // Gram and residual sums sit in the reduction record between the steps
   b.finalize = p->sharded ? 1 : 0;

@@ -29,7 +29,7 @@ constexpr int kMaxTW = 224;          // largest frame count of the wide (shared-
 constexpr int kPassThreads = 256;    // one pixel per thread per tile
 constexpr int kTile = kPassThreads;  // pixels per CTA tile
 constexpr int kPassCtasPerSm = 1;    // resident CTAs of the narrow passes per SM
-constexpr int kGroup = 16;           // CTAs per first-level reduction group
+constexpr int kGroup = 16;           // CTAs per first-level reduction group (narrow windows, batches)
 constexpr int kMaxGroups = 64;
 
 // Pass kinds.
@@ -141,6 +141,7 @@ struct Bufs {
   int T;
   int grid;
   int ngroups;
+  int group;           // CTAs per first-level reduction group
   int cplx;            // complex window: T = 2 x frames, columns (2t, 2t + 1) = (Re, Im) of frame t
   int wide;            // tiled path: the reduced Gram goes to Gw (T x T), else to red->G (kMaxT stride)
   int finalize;        // 1: the pass itself sums the group partials into red->G, e2, l1;

@@ -210,6 +210,7 @@ static __device__ __noinline__ int eig_wide_factor(float* W, int T, EigWideSh& S
   if (r2 <= 2) jac_cholesky<1>(W, LD, T, S.diag, S.piv);
   else if (r2 <= 4) jac_cholesky<2>(W, LD, T, S.diag, S.piv);
   else if (r2 <= 8) jac_cholesky<4>(W, LD, T, S.diag, S.piv);
+  else if (r2 <= 10) jac_cholesky<5>(W, LD, T, S.diag, S.piv);
   else jac_cholesky<7>(W, LD, T, S.diag, S.piv);
   switch (r2) {
 #define RPCA_JAC(R) \
@@ -245,7 +246,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
     if (b.finalize) {
       for (int e = e0 + i; e < e1; e += n) G[e / T * ld + e % T] = (float)__ldcg(&b.Gw[e]);
     } else if (__ldcg(&b.red->gram_last)) {
-      sum_rows<4>(b.group_part, 0, __ldcg(&b.red->ngroups_last), TT,
+      sum_rows<4, 8>(b.group_part, 0, __ldcg(&b.red->ngroups_last), TT,
                   [&](int e, float gh, float gl) { G[e / T * ld + e % T] = gh + gl; }, i, n, e0, e1);
     }
   };
@@ -554,7 +555,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   if (lane == 0) S.perm[warp] = kept;
   if (b.wtc) {
     eig_sync(nr);  // Ww and Vw written by every rank
-    if (rank == 0) wtc_images(b);
+    wtc_images(b, M(ES_VT), ld, rank, nr);
   } else {
     __syncthreads();
   }

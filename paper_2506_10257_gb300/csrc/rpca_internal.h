@@ -43,10 +43,10 @@ size_t wide_tc_img_bytes(int T, int precision);
 // Fills *out for T real columns (complex windows: T = 2 x frames, cplx set);
 // false when T is not a wide column count (real T <= kMaxT unless force) or a
 // kernel attribute cannot be set.
-bool wide_kernels(int T, bool cplx, bool force, WideKernels* out);
+bool wide_kernels(int T, bool cplx, bool force, int64_t m, int sms, WideKernels* out);
 
-// Pixels per tile and CTAs per SM of the tiled pass for T real columns.
-void wide_launch_shape(int T, int* tile, int* per_sm);
+// Pixels per tile and CTAs per SM of the tiled pass for T real columns and m pixels.
+void wide_launch_shape(int T, bool cplx, int64_t m, int sms, int* tile, int* per_sm);
 
 // rpca_plan_create with the tiled path forced for any frame count (the
 // batched form runs every window of a batch that holds a wide or complex

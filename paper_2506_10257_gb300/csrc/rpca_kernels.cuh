@@ -187,29 +187,29 @@ __device__ __forceinline__ float2 ff_term(float2 v) { return v; }
 // Sums rows [r0, r1) of entries [e0, e1) (all by default) of a row-major [rows][TT] array (FP32 partials of the
 // CTAs, or two-float group sums) entry by entry in two-float arithmetic in a
 // fixed row order, calling out(e, hi, lo) for every entry; each thread takes
-// entries tid, tid + blockDim, ... and issues its loads in batches of 16 so
+// entries tid, tid + blockDim, ... and issues its loads R rows at a time so
 // that their L2 latencies overlap.  The reduced Gram thus carries only the
 // rounding of the CTAs' own FP32 accumulations.
-template <int W = 1, typename Src, typename Out>
+template <int W = 1, int R = 16, typename Src, typename Out>
 __device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT, Out out, int tid = threadIdx.x,
                                          int nthr = blockDim.x, int e0 = 0, int e1 = -1) {
-  // W = 4: four entries per step (T x T Grams of wide windows), so that 64
+  // W = 4: four entries per step (T x T Grams of wide windows), so that 4 R
   // loads are in flight per thread
   if (e1 < 0) e1 = TT;
   int e = e0 + tid;
   for (; W == 4 && e + 3 * nthr < e1; e += 4 * nthr) {
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int rb = r0; rb < r1; rb += 16) {
-      Src v[4][16];
+    for (int rb = r0; rb < r1; rb += R) {
+      Src v[4][R];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
+        for (int u = 0; u < R; ++u)
           v[q][u] = (rb + u < r1) ? __ldcg(&src[(int64_t)(rb + u) * TT + e + q * nthr]) : Src{};
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < R; ++u) {
           const float2 t = ff_term(v[q][u]);  // (zero past the last row)
           ff_add(h[q], l[q], t.x, t.y);
         }
@@ -219,12 +219,12 @@ __device__ __forceinline__ void sum_rows(const Src* src, int r0, int r1, int TT,
   }
   for (; e < e1; e += nthr) {
     float h = 0.f, l = 0.f;
-    for (int rb = r0; rb < r1; rb += 16) {
-      Src v[16];
+    for (int rb = r0; rb < r1; rb += R) {
+      Src v[R];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = (rb + u < r1) ? __ldcg(&src[(int64_t)(rb + u) * TT + e]) : Src{};
+      for (int u = 0; u < R; ++u) v[u] = (rb + u < r1) ? __ldcg(&src[(int64_t)(rb + u) * TT + e]) : Src{};
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
+      for (int u = 0; u < R; ++u) {
         const float2 t = ff_term(v[u]);  // (zero past the last row)
         ff_add(h, l, t.x, t.y);
       }
@@ -265,7 +265,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 
 // Reduction across the nc CTAs of a pass (this one is number lc) after every
 // CTA wrote its partial Gram (gram_part) and scalar sums (scal_part): the last
-// CTA of each group of kGroup sums its group, the last group reducer sums the
+// CTA of each group of b.group sums its group, the last group reducer sums the
 // groups, in fixed order, into red->G, red->e2 and red->l1 (only when
 // b.finalize; otherwise the next eigen-step does).  Called by all threads of
 // every CTA; returns true in the CTA that wrote the final sums.
@@ -275,12 +275,12 @@ static __device__ __noinline__ bool cross_cta_reduce(Bufs b, bool kGram, double*
   const int T = b.T;
   const int TT = T * T;
   int& sLast = *sLastp;
-  // ---- level 1: last CTA of each group of kGroup CTAs ----
+  // ---- level 1: last CTA of each group of CTAs ----
   __threadfence();
   __syncthreads();
-  const int grp = lc / kGroup;
-  const int c0 = grp * kGroup;
-  const int c1 = min(c0 + kGroup, nc);
+  const int grp = lc / b.group;
+  const int c0 = grp * b.group;
+  const int c1 = min(c0 + b.group, nc);
   if (tid == 0) {
     atomicMax(&b.red->t_loop, gtimer());
     const unsigned t = atomicAdd(&b.red->cnt[grp], 1u);
@@ -291,7 +291,7 @@ static __device__ __noinline__ bool cross_cta_reduce(Bufs b, bool kGram, double*
   __threadfence();
   if (kGram) {
     float2* gp = b.group_part + (int64_t)grp * TT;
-    sum_rows<W>(b.gram_part, c0, c1, TT, [&](int e, float h, float l) { gp[e] = make_float2(h, l); });
+    sum_rows<W, W == 1 ? 16 : 4>(b.gram_part, c0, c1, TT, [&](int e, float h, float l) { gp[e] = make_float2(h, l); });
   }
   sum_scalars(b.scal_part, c0, c1, sScal, [&](double s0, double s1) {
     b.gscal_part[2 * grp] = s0;
@@ -299,7 +299,7 @@ static __device__ __noinline__ bool cross_cta_reduce(Bufs b, bool kGram, double*
     b.red->cnt[grp] = 0u;
     atomicMax(&b.red->t_l1, gtimer());
   });
-  const int ngroups = (nc + kGroup - 1) / kGroup;
+  const int ngroups = (nc + b.group - 1) / b.group;
   if (!b.finalize) {
     // the next eigen-step sums the group partials
     if (tid == 0) {

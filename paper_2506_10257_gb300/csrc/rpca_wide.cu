@@ -6,29 +6,15 @@
 
 namespace rpca {
 
-template <int CW, bool CPLX>
+template <int TP, int RP, bool CPLX>
 WideKernels make_wide() {
-  constexpr int TP = 8 * CW;
   WideKernels k;
-  if constexpr (TP <= 128) {
-    // Wbar and V resident in shared memory, 64-pixel tiles
-    k.pass[PM_INIT] = (void*)pass_res_kernel<TP, PM_INIT, CPLX>;
-    k.pass[PM_FUSED] = (void*)pass_res_kernel<TP, PM_FUSED, CPLX>;
-    k.pass[PM_UPDATE] = (void*)pass_res_kernel<TP, PM_UPDATE, CPLX>;
-    k.pass[PM_GRAM] = (void*)pass_res_kernel<TP, PM_GRAM, CPLX>;
-    k.pass_smem = res_pass_smem_bytes(TP);
-    k.tile = kRP;
-    k.per_sm = res_blocks_per_sm(TP);
-  } else {
-    // Wbar and V streamed 32 rows at a time, 32-pixel tiles
-    k.pass[PM_INIT] = (void*)pass_wide_kernel<CW, PM_INIT, CPLX>;
-    k.pass[PM_FUSED] = (void*)pass_wide_kernel<CW, PM_FUSED, CPLX>;
-    k.pass[PM_UPDATE] = (void*)pass_wide_kernel<CW, PM_UPDATE, CPLX>;
-    k.pass[PM_GRAM] = (void*)pass_wide_kernel<CW, PM_GRAM, CPLX>;
-    k.pass_smem = WideShape<CW>::smem;
-    k.tile = kWP;
-    k.per_sm = 1;
-  }
+  k.pass[PM_INIT] = (void*)pass_tile_kernel<TP, RP, PM_INIT, CPLX>;
+  k.pass[PM_FUSED] = (void*)pass_tile_kernel<TP, RP, PM_FUSED, CPLX>;
+  k.pass[PM_UPDATE] = (void*)pass_tile_kernel<TP, RP, PM_UPDATE, CPLX>;
+  k.pass[PM_GRAM] = (void*)pass_tile_kernel<TP, RP, PM_GRAM, CPLX>;
+  k.tile = RP;
+  k.per_sm = tile_blocks_per_sm(TP, CPLX);
   k.pass_threads = kWideThreads;
   k.eig = (void*)eig_wide_kernel;
   k.eig_threads = kEigWThreads;
@@ -60,31 +46,27 @@ size_t wide_tc_img_bytes(int T, int precision) {
   return 0;
 }
 
-void wide_launch_shape(int T, int* tile, int* per_sm) {
-  const int TP = (T + 31) / 32 * 32;
-  *tile = TP <= 128 ? kRP : kWP;
-  *per_sm = TP <= 128 ? res_blocks_per_sm(TP) : 1;
+void wide_launch_shape(int T, bool cplx, int64_t m, int sms, int* tile, int* per_sm) {
+  *tile = tile_rp(T, cplx, m, sms);
+  *per_sm = tile_blocks_per_sm(tile_tp(T, cplx), cplx);
 }
 
-template <bool CPLX>
-WideKernels pick_wide(int TP) {
-  switch (TP) {
-    case 32: return make_wide<4, CPLX>();
-    case 64: return make_wide<8, CPLX>();
-    case 96: return make_wide<12, CPLX>();
-    case 128: return make_wide<16, CPLX>();
-    case 160: return make_wide<20, CPLX>();
-    case 192: return make_wide<24, CPLX>();
-    default: return make_wide<28, CPLX>();
-  }
-}
-
-bool wide_kernels(int T, bool cplx, bool force, WideKernels* out) {
+bool wide_kernels(int T, bool cplx, bool force, int64_t m, int sms, WideKernels* out) {
   if (T > kMaxTW || T < 1) return false;
   if (!cplx && T <= kMaxT && !force) return false;
   if (cplx && (T & 1)) return false;
-  const int TP = (T + 31) / 32 * 32;
-  *out = cplx ? pick_wide<true>(TP) : pick_wide<false>(TP);
+  const int RP = tile_rp(T, cplx, m, sms);
+  switch (tile_tp(T, cplx)) {
+    case 32: *out = cplx ? make_wide<32, 128, true>() : make_wide<32, 128, false>(); break;
+    case 64: *out = cplx ? make_wide<64, 128, true>() : RP == 64 ? make_wide<64, 64, false>() : make_wide<64, 128, false>(); break;
+    case 96: *out = cplx ? make_wide<96, 128, true>() : RP == 64 ? make_wide<96, 64, false>() : make_wide<96, 128, false>(); break;
+    case 128: *out = cplx ? make_wide<128, 128, true>() : RP == 64 ? make_wide<128, 64, false>() : make_wide<128, 128, false>(); break;
+    case 160: *out = make_wide<160, 64, false>(); break;
+    case 192: *out = cplx ? make_wide<192, 64, true>() : make_wide<192, 64, false>(); break;
+    case 224: *out = make_wide<224, 64, false>(); break;
+    default: *out = make_wide<256, 64, true>(); break;
+  }
+  out->pass_smem = tile_pass_smem(T, RP, cplx);
   // the sweeps' columns, or one rank's operands of a product, as far as they fit
   const size_t ops = 2 * sizeof(float) * (size_t)T * (eig_ld(T) + (eig_ld(T) / 4 + kEigWRanks - 1) / kEigWRanks * 4);
   out->eig_smem = eig_wide_smem(T);

@@ -114,14 +114,14 @@ __device__ __forceinline__ void tc_store1(unsigned char* hi, unsigned char* lo, 
 // CTA after it has written Ww and Vw): image [m][c] holds rows n < TP and
 // frames k of chunk c of B[n][k] = M[k][n] (M = Wbar or V), zero outside T.
 template <int TP, bool BF16>
-__device__ void wtc_write_images(const Bufs& b) {
+__device__ void wtc_write_images(const Bufs& b, const float* vt, int ldv, int rank, int nr) {
   using SH = WtcShape<TP, BF16>;
   const int T = b.T;
-  for (int i = threadIdx.x; i < 2 * TP * TP; i += blockDim.x) {
+  for (int i = threadIdx.x + rank * blockDim.x; i < 2 * TP * TP; i += nr * blockDim.x) {
     const int mat = i / (TP * TP), e = i % (TP * TP);
     const int n = e / TP, k = e % TP;
-    const float* M = mat ? b.Vw : b.Ww;
-    const float v = (n < T && k < T) ? __ldcg(&M[k * T + n]) : 0.f;
+    // (row n of V^T, and of Wbar, which is symmetric: consecutive k)
+    const float v = (n < T && k < T) ? __ldcg(mat ? &vt[n * ldv + k] : &b.Ww[n * T + k]) : 0.f;
     const int c = k / kWtcKCh;
     unsigned char* hi = b.wtc_img + ((size_t)(mat * SH::NCH + c) * 2) * SH::B_BYTES;
     tc_store1<BF16>(hi, hi + SH::B_BYTES, SH::off(n, k % kWtcKCh), v);
