@@ -330,7 +330,9 @@ static cudaError_t add_kernel(cudaGraph_t g, cudaGraphNode_t* node, const cudaGr
   return cudaGraphAddKernelNode(node, g, deps, ndeps, &kp);
 }
 
-// Graph: init pass -> eig(init) -> while(cond){ fused pass -> eig(check|eig) } -> final.
+// Graph: init pass -> eig(init) -> while(cond){ (fused pass -> eig(check|eig)) x kLoopUnroll } -> final.
+constexpr int kLoopUnroll = 4;
+
 static rpca_status build_graph(rpca_plan_s* pl) {
   CK(cudaGraphCreate(&pl->graph, 0));
   cudaGraphConditionalHandle h;
@@ -367,8 +369,13 @@ static rpca_status build_graph(rpca_plan_s* pl) {
   cp.conditional.size = 1;
   CK(cudaGraphAddNode(&n_while, pl->graph, &n_eig0, nullptr, 1, &cp));
   cudaGraph_t body = cp.conditional.phGraph_out[0];
-  CK(add_kernel(body, &n_pass, nullptr, 0, fused_fn(pl), fused_grid(pl), fused_block(pl), a_pass, fused_smem(pl)));
-  CK(add_kernel(body, &n_eig, &n_pass, 1, eig_fn(pl), eg, eb, a_eig1, es));
+  // kLoopUnroll iterations per evaluation of the loop condition, which costs about
+  // as much as two launches; iterations after the last one return at once.
+  for (int it = 0; it < kLoopUnroll; ++it) {
+    CK(add_kernel(body, &n_pass, it ? &n_eig : nullptr, it ? 1 : 0, fused_fn(pl), fused_grid(pl), fused_block(pl), a_pass,
+                  fused_smem(pl)));
+    CK(add_kernel(body, &n_eig, &n_pass, 1, eig_fn(pl), eg, eb, a_eig1, es));
+  }
 
   const int fgrid = (int)std::min<int64_t>((pl->p.m + 255) / 256, 4096);
   CK(add_kernel(pl->graph, &n_fin, &n_while, 1, (void*)final_kernel, dim3(fgrid), dim3(256), a_pass));
