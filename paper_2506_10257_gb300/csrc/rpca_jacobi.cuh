@@ -209,79 +209,78 @@ static __device__ __noinline__ int jac_sweeps(float* W, int LD, int nb, float* n
   return sweep;
 }
 
-// Cholesky factor of the matrix whose lower triangle is in W (column j at
-// W + j LD, entry i at + i; zero elsewhere, and zero beyond T), in place, four
-// columns at a time: warp 0 factors a panel in registers (lane = row), then all
-// warps update the columns after it.  A pivot below kJacFloor times its diagonal
-// entry diag[j] (a numerically dependent column, or one of a block that rounding
-// left indefinite) is raised to that and the rest of its column dropped, so that
-// the columns stay independent and bounded.  piv: T floats of scratch.  RU: rows / 32 rounded up.
-// All threads call it after a barrier; it ends with one.
-template <int RU>
-static __device__ __noinline__ void jac_cholesky(float* W, int LD, int T, const float* diag, float* piv) {
-  __builtin_assume(__isShared(W));
-  __builtin_assume(__isShared(diag));
-  __builtin_assume(__isShared(piv));
+// The panels of four columns in rows 32 UB .. 32 UB + 31, and what they change
+// beyond; rows 32 u + lane, u in [UB, RU), so the row groups above are left out at
+// compile time.  v: warp 0's current panel (set by the caller for column 0).
+template <int RU, int UB>
+__device__ __forceinline__ void jac_chol_rows(float* W, int LD, int T, const float* diag, float* piv, float (&v)[4][RU]) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int j0 = 0; j0 < T; j0 += 4) {
-    const int jn = min(4, T - j0);
+#pragma unroll 1
+  for (int j0 = 32 * UB; j0 < min(32 * UB + 32, T); j0 += 4) {
+    const int l0 = j0 - 32 * UB;  // lane of the panel's first row
     if (warp == 0) {
-      float v[4][RU];
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int u = 0; u < RU; ++u) {
-          const int i = j0 + lane + 32 * u;
-          v[c][u] = (c < jn && i < T) ? W[(j0 + c) * LD + i] : 0.f;
-        }
+      // factor the panel in registers
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        if (c >= jn) break;
-        const float raw = __shfl_sync(full, v[c][0], c), floor = fmaxf(kJacFloor * diag[j0 + c], 1e-30f);
+        const bool in = j0 + c < T;
+        const float raw = __shfl_sync(full, v[c][UB], l0 + c), floor = in ? fmaxf(kJacFloor * diag[j0 + c], 1e-30f) : 1.f;
         const float pv = fmaxf(raw, floor);
         if (!(raw > floor)) {
 #pragma unroll
-          for (int u = 0; u < RU; ++u) v[c][u] = 0.f;
+          for (int u = UB; u < RU; ++u) v[c][u] = 0.f;
         }
-        if (lane == c) v[c][0] = pv;
-        if (lane == 0) piv[j0 + c] = pv;
+        if (lane == l0 + c) v[c][UB] = pv;
+        if (lane < l0 + c) v[c][UB] = 0.f;
+        if (lane == 0 && in) piv[j0 + c] = pv;
         const float rd = __fdividef(1.f, pv);
 #pragma unroll
         for (int e = c + 1; e < 4; ++e) {
-          const float f = __shfl_sync(full, v[c][0], e) * rd;
+          const float f = __shfl_sync(full, v[c][UB], l0 + e) * rd;
 #pragma unroll
-          for (int u = 0; u < RU; ++u) v[e][u] = fmaf(-f, v[c][u], v[e][u]);
+          for (int u = UB; u < RU; ++u) v[e][u] = fmaf(-f, v[c][u], v[e][u]);
         }
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int u = 0; u < RU; ++u) {
-          const int i = j0 + lane + 32 * u;
-          if (c < jn && i < T) W[(j0 + c) * LD + i] = (lane + 32 * u >= c) ? v[c][u] : 0.f;
-        }
+        for (int u = UB; u < RU; ++u)
+          if (j0 + c < T && 32 * u + lane < T) W[(j0 + c) * LD + 32 * u + lane] = v[c][u];
     }
     __syncthreads();
-    if (j0 + 4 < T) {
-      // lane = row (from j0 + 4 on); the panel's rows stay in registers over the columns
-      float rd[4], w[4][RU];
+    if (j0 + 4 >= T) break;
+    // the columns after the panel: warp 0 takes the next panel and keeps it, the
+    // others the rest (their updates are done by the next barrier)
+    float rd[4], w[4][RU];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        rd[c] = __fdividef(1.f, piv[j0 + c]);
+    for (int c = 0; c < 4; ++c) {
+      rd[c] = __fdividef(1.f, piv[j0 + c]);
 #pragma unroll
-        for (int u = 0; u < RU; ++u) {
-          const int i = j0 + 4 + lane + 32 * u;
-          w[c][u] = i < T ? W[(j0 + c) * LD + i] : 0.f;
+      for (int u = UB; u < RU; ++u) w[c][u] = warp == 0 ? v[c][u] : 32 * u + lane < T ? W[(j0 + c) * LD + 32 * u + lane] : 0.f;
+    }
+    if (warp == 0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = j0 + 4 + e;
+        float f[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) f[c] = k < T ? -rd[c] * W[(j0 + c) * LD + k] : 0.f;
+#pragma unroll
+        for (int u = UB; u < RU; ++u) {
+          float x = k < T && 32 * u + lane < T ? W[k * LD + 32 * u + lane] : 0.f;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) x = fmaf(f[c], w[c][u], x);
+          v[e][u] = x;
         }
       }
-      for (int k = j0 + 4 + warp; k < T; k += nwarps) {
+    } else {
+      for (int k = j0 + 8 + warp - 1; k < T; k += nwarps - 1) {
         float f[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) f[c] = -rd[c] * W[(j0 + c) * LD + k];
 #pragma unroll
-        for (int u = 0; u < RU; ++u) {
-          const int i = j0 + 4 + lane + 32 * u;
+        for (int u = UB; u < RU; ++u) {
+          const int i = 32 * u + lane;
           if (i >= k && i < T) {
             float x = W[k * LD + i];
 #pragma unroll
@@ -293,6 +292,37 @@ static __device__ __noinline__ void jac_cholesky(float* W, int LD, int T, const 
     }
     __syncthreads();
   }
+}
+template <int RU, int UB = 0>
+__device__ __forceinline__ void jac_chol_all(float* W, int LD, int T, const float* diag, float* piv, float (&v)[4][RU]) {
+  if constexpr (UB < RU) {
+    jac_chol_rows<RU, UB>(W, LD, T, diag, piv, v);
+    jac_chol_all<RU, UB + 1>(W, LD, T, diag, piv, v);
+  }
+}
+
+// Cholesky factor of the matrix whose lower triangle is in W (column j at
+// W + j LD, entry i at + i; zero elsewhere, and zero beyond T), in place, four
+// columns at a time: warp 0 factors a panel in registers (lane = row), then all
+// warps update the columns after it, warp 0 those of the next panel.  A pivot
+// below kJacFloor times its diagonal entry diag[j] (a numerically dependent
+// column, or one of a block that rounding left indefinite) is raised to that and
+// the rest of its column dropped, so that the columns stay independent and
+// bounded.  piv: T floats of scratch.  RU: rows / 32 rounded up.  At least two
+// warps; all threads call it after a barrier; it ends with one.
+template <int RU>
+static __device__ __noinline__ void jac_cholesky(float* W, int LD, int T, const float* diag, float* piv) {
+  __builtin_assume(__isShared(W));
+  __builtin_assume(__isShared(diag));
+  __builtin_assume(__isShared(piv));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  float v[4][RU];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int u = 0; u < RU; ++u) v[c][u] = warp == 0 && c < T && 32 * u + lane < T ? W[c * LD + 32 * u + lane] : 0.f;
+  jac_chol_all<RU>(W, LD, T, diag, piv, v);
+  __syncthreads();
   for (int j = warp; j < T; j += nwarps) {
     const float r = rsqrtf(piv[j]);
     for (int i = j + lane; i < T; i += 32) W[j * LD + i] *= r;
