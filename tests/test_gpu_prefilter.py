@@ -169,3 +169,39 @@ def test_highpass_rejects_bad_arguments(rp):
     X = torch.zeros((4, 64), dtype=torch.float32, device="cuda")
     with pytest.raises(rp.RpcaError):
         rp.prefilter(X, window=0, high_pass=True)
+
+
+@pytest.mark.parametrize("high_pass", [False, True])
+@pytest.mark.parametrize("kind", ["large", "infinite", "cancelling"])
+def test_moving_average_beyond_the_range_of_two_float_sums(rp, kind, high_pass):
+    # sums that leave FP32's range (or are not finite) fall back to FP64 sums; sums of
+    # opposite signs keep what FP32 sums would lose
+    rng = np.random.Generator(np.random.PCG64(3))
+    F = (1.0 + 0.1 * rng.standard_normal((40, 300))).astype(np.float32)
+    F[:, :] += F[0]
+    if kind == "large":
+        F[:, 100:200] *= np.float32(1e38)
+    elif kind == "infinite":
+        F[20, 7] = np.inf
+    else:
+        F[::2, 50:90] += np.float32(3e7)
+        F[1::2, 50:90] -= np.float32(3e7)
+    X = torch.from_numpy(F).cuda()
+    Y, kept, _ = rp.prefilter(X, corr_min=-2.0, window=20, high_pass=high_pass)
+    G = F[kept.cpu().numpy()].astype(np.float64)
+    with np.errstate(invalid="ignore"):
+        # slid as the kernel slides: a sum that was infinite once is not a number afterwards
+        ref = []
+        for j0 in range(0, len(G) - 19, 16):
+            s = G[j0:j0 + 20].sum(0)
+            for j in range(j0, min(j0 + 16, len(G) - 19)):
+                if j > j0:
+                    s = s + G[j + 19] - G[j - 1]
+                ref.append(G[j + 9] - s / 20 if high_pass else s / 20)
+        ref = np.array(ref)
+    got = Y.cpu().numpy().astype(np.float64)
+    fine = np.isfinite(ref)
+    assert (np.isfinite(got) == fine).all() and (np.isnan(got) == np.isnan(ref)).all()
+    # one FP32 rounding of the result, and of the mean where the centre frame is subtracted exactly
+    scale = np.abs(G).max(0)
+    assert (np.abs(got - ref)[fine] <= (2.0 ** -23 * np.abs(ref) + 2.0 ** -40 * scale)[fine]).all()
