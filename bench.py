@@ -318,7 +318,7 @@ def _eig_desc() -> str:
 def _plan_pass_name(T, m, args):
     """The fused pass kernel a plan runs (the rule of the plan's kernel choice)."""
     if args.complex or T > 32:
-        return "pass_res_kernel / pass_wide_kernel (tiled, FUSED)"
+        return "pass_tile_kernel (tiled, FUSED)"
     tb = next(b for b in (8, 12, 16, 20, 24, 32) if T <= b)
     if args.precision != "fp32":
         return f"pass_tc_kernel ({args.precision}, tcgen05)"

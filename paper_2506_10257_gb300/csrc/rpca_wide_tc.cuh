@@ -2,7 +2,7 @@
 // with all three dense contractions on the 5th-generation tensor cores
 // (included inside namespace rpca by rpca_wide.cuh).
 //
-// Same iteration as pass_res_body (Eq. 4-6 through the Gram of Z, the residual
+// Same iteration as pass_tile_body (Eq. 4-6 through the Gram of Z, the residual
 // of Sec. II-A and the rotated Gram of the next Z), arranged for tcgen05:
 //   Q  = Z Wbar       (128-pixel tile x TP columns, K = TP frames)
 //   Z~ = Z' V         (the next iteration's Z in the current eigenbasis)
