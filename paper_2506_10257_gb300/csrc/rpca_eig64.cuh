@@ -22,8 +22,8 @@
 // and the sweeps stop once what is neglected on the former is below the result's
 // FP32 rounding.  A step that finds more left there runs another round of sweeps
 // on diag(d) + E.  sigma, the sigma > tau decision, g and mu are FP64.  Measured on
-// the windows above: 30 us (load 3, factor and sweeps 18, products and decisions 9)
-// and 52 us, at the same errors of L and S against 64 bits (1.0e-7 and 2.3e-7).
+// the windows above: 25 us (load 3, factor and sweeps 13, products and decisions 10)
+// and 44 us, at the same errors of L and S against 64 bits (1.0e-7 and 2.3e-7).
 #pragma once
 
 constexpr int kEigThreads = 256;   // threads of the eigen-step CTA

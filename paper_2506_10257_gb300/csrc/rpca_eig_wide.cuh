@@ -20,8 +20,11 @@
 // rank 0 factors and sweeps with the matrix in its shared memory; the Gram's
 // cross-CTA sums and the five T x T x T products are spread over the ranks by
 // rows, with every T x T operand in the workspace (L2) and a cluster barrier
-// between products.  A single SM would need as long for the products as for the
-// sweeps, and several times as long to read the partial Grams.
+// between products.  Bound by the factor and the sweeps on rank 0's SM, which wait
+// at its barriers.  Measured with 8 ranks, against cyclic Jacobi on the Gram itself:
+// 50 frames 295 -> 118 us (factor and sweeps 47, products 47), 100 frames
+// 1106 -> 273 us (170, 63), 132 frames 2310 -> 491 us (353, 92).  One CTA, beside
+// the other lanes of a batch, takes 220 us at 63 frames and 405 us at 93.
 #pragma once
 
 // Matrices of the step's scratch, each eig_ld(T)^2 floats.

@@ -24,6 +24,9 @@
 // 64-pixel tiles.  What bounds the pass is the FP32 pipe: per k a thread loads one
 // 16-byte group of Z (four in a warp) and CPT values of Wbar or V (eight groups in a
 // warp, each a conflict-free 16-byte load) for 4 CPT multiply-adds.
+// Measured, with the tile that held S and Y -> now: 262144 x 50 248 -> 192 us (FMA pipe
+// 33 % busy, most stalls on shared memory), 87880 x 132 760 -> 430 us, complex
+// 65536 x 50 331 -> 261 us.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
