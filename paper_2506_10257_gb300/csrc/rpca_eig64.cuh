@@ -144,6 +144,7 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
   const unsigned long long t1 = gtimer();
   unsigned long long t2 = t1, t3 = t1;
   int sweeps = 0;
+  const double mu_prev = init ? __ldcg(&ctrl->mu_cur) : 0.0;  // (of the plan's previous solve)
   for (int pass = 0;; ++pass) {
     // ---- descending order of the diagonal; Cholesky factor; one-sided Jacobi ----
     // (every warp works the order out and writes the same values)
@@ -237,7 +238,7 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
     if (init && tid == 0) {
       double lmax = 0.0;
       for (int a = 0; a < T; ++a) lmax = fmax(lmax, S.d[a]);
-      init_mu(b, lmax / (double)scale);
+      init_mu(b, lmax / (double)scale, mu_prev);
       sTau = ctrl->inv_cur;
     }
     if (init) __syncthreads();

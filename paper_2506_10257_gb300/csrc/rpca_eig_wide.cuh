@@ -274,6 +274,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   float scale = 1.f, rootf = 1.f;
   int sweeps = 0;
   double tau = init ? 0.0 : __ldcg(&ctrl->inv_cur);
+  const double mu_prev = init ? __ldcg(&ctrl->mu_cur) : 0.0;  // (of the plan's previous solve)
   float tauf = 0.f;
   for (int pass = 0;; ++pass) {
     if (rank == 0) {
@@ -432,7 +433,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       if (rank == 0 && tid == 0) {
         double lmax = 0.0;
         for (int a = 0; a < T; ++a) lmax = fmax(lmax, S.d[a]);
-        init_mu(b, lmax / (double)scale);
+        init_mu(b, lmax / (double)scale, mu_prev);
       }
       eig_sync(nr);
       tau = __ldcg(&ctrl->inv_cur);

@@ -816,9 +816,11 @@ __device__ __forceinline__ void refresh_next(Ctrl* c) {
 // First mu of a solve (FP64, thread 0 of an eigen-step with EF_INIT): the
 // schedule's mu0 (Sec. II-A: 1.25/||X||_2 from the top Gram eigenvalue lmax,
 // or m T / (4 ||X||_1)), unless the plan sets mu_init, or asks a warm start to
-// resume from mu_prev_scale times its previous solve's final mu.  The cap
-// mu_max = mu_max_factor * mu0 always follows the cold schedule.
-__device__ __forceinline__ void init_mu(Bufs b, double lmax) {
+// resume from mu_prev_scale times its previous solve's final mu, mu_prev (the
+// caller reads it before the first call: a step of several rounds calls this in
+// each, with the eigenvalue of that round).  The cap mu_max = mu_max_factor * mu0
+// always follows the cold schedule.
+__device__ __forceinline__ void init_mu(Bufs b, double lmax, double mu_prev) {
   Ctrl* c = b.ctrl;
   const double frames = b.cplx ? 0.5 * (double)b.T : (double)b.T;  // n1 n2 counts complex entries once
   const double mu0 = (c->schedule == 0) ? c->mu0_scale / sqrt(lmax)
@@ -826,8 +828,8 @@ __device__ __forceinline__ void init_mu(Bufs b, double lmax) {
   double mu1 = mu0;
   if (c->mu_init > 0.0)
     mu1 = c->mu_init;
-  else if (c->warm && c->mu_prev_scale > 0.0 && c->mu_cur > 0.0)
-    mu1 = c->mu_prev_scale * c->mu_cur;
+  else if (c->warm && c->mu_prev_scale > 0.0 && mu_prev > 0.0)
+    mu1 = c->mu_prev_scale * mu_prev;
   c->mu_cur = mu1;
   c->mu_max = c->mu_max_factor * mu0;
   c->mu_nxt = (c->schedule == 0) ? fmin(c->rho * mu1, c->mu_max) : mu1;
