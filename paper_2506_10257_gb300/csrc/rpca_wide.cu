@@ -1,6 +1,8 @@
 // rpca_wide.cu -- host side of the wide / complex path: kernel tables.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "rpca_internal.h"
 #include "rpca_wide.cuh"
 
@@ -71,11 +73,14 @@ bool wide_kernels(int T, bool cplx, bool force, int64_t m, int sms, WideKernels*
   const size_t ops = 2 * sizeof(float) * (size_t)T * (eig_ld(T) + (eig_ld(T) / 4 + kEigWRanks - 1) / kEigWRanks * 4);
   out->eig_smem = eig_wide_smem(T);
   if (ops > out->eig_smem) out->eig_smem = ops < kEigWMaxSmem ? ops : (out->eig_smem > kEigWMaxSmem ? out->eig_smem : kEigWMaxSmem);
-  if (cudaFuncSetAttribute(out->eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out->eig_smem) != cudaSuccess)
+  // The kernels are shared by plans of other frame counts, which may have been made before and launch with their own
+  // size: the limits are those of the largest one, whatever this plan needs.
+  static_assert(eig_wide_smem(kMaxTW) <= kEigWMaxSmem, "the sweeps of the longest columns fit");
+  const int pass_max = (int)tile_pass_smem(std::min(tile_tp(T, cplx), kMaxTW), RP, cplx);
+  if (cudaFuncSetAttribute(out->eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEigWMaxSmem) != cudaSuccess)
     return false;
   for (int i = 0; i < 4; ++i)
-    if (cudaFuncSetAttribute(out->pass[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out->pass_smem) !=
-        cudaSuccess)
+    if (cudaFuncSetAttribute(out->pass[i], cudaFuncAttributeMaxDynamicSharedMemorySize, pass_max) != cudaSuccess)
       return false;
   for (int i = 0; i < 4; ++i)
     if (out->pass_tc[i] && cudaFuncSetAttribute(out->pass_tc[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
