@@ -467,7 +467,8 @@ rpca_status rpca_step_done(rpca_plan_t plan, int32_t* done, rpca_result* out, vo
  *   scratch device memory of rpca_prefilter_scratch_bytes(m, T) bytes, owned by
  *           the caller, not shared with a call in flight.
  * Correlations are accumulated in FP64 (FP32 inputs make every product exact);
- * the window sums slide as two-float pairs (FP64 where they leave FP32's range).  Errors: RPCA_ERR_ARG (a null pointer, m < 1,
+ * the window sums slide as three floats, which carry more than FP64 does (FP64
+ * where they leave FP32's range).  Errors: RPCA_ERR_ARG (a null pointer, m < 1,
  * T < 1, window < 1, corr_min NaN, X or Y not 4-byte aligned),
  * RPCA_ERR_UNSUPPORTED (T > 65535), RPCA_ERR_CUDA (a launch failed).  The
  * outputs are valid once `stream` has reached the call. */

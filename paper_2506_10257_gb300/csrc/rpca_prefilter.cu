@@ -18,13 +18,15 @@
 //   pf_decide_kernel  one CTA: sums the chunks in fixed order, forms the
 //                     neighbour correlations, keeps frames, writes the counts;
 //   pf_average_kernel a thread per (pixel, 16 output frames): the window sum
-//                     as a two-float (hi, lo) pair on the FP32 pipe, formed
-//                     directly for the first output and slid for the rest
-//                     (exact for FP32 inputs of similar magnitude), each output
-//                     frame rounded once to FP32.  FP64 sums, at 1/64 of the FP32
-//                     rate, bound it (87880 pixels x 132 frames, the whole
-//                     pre-filter: 466 us, now 346); they remain for segments whose
-//                     sums leave FP32's range (large or non-finite inputs).
+//                     as three floats on the FP32 pipe, formed directly for the
+//                     first output and slid for the rest (exact for FP32 inputs of
+//                     similar magnitude), each output frame rounded once to FP32.
+//                     Three floats carry about 2^-72 of the largest partial sum,
+//                     FP64 2^-53, a (hi, lo) pair only 2^-48, which shows where large
+//                     frames of opposite sign cancel or slide out.  FP64 sums, at
+//                     1/64 of the FP32 rate, bound it (87880 pixels x 132 frames, the
+//                     whole pre-filter: 411 us, now 310); they remain for segments whose sums
+//                     leave FP32's range (very large, very small or non-finite inputs).
 //
 // The temporal high-pass that Sec. IV suggests before RPCA (no filter is
 // defined there) is read as the complement of the same moving average: output
@@ -139,14 +141,30 @@ __global__ void __launch_bounds__(kPfThreads) pf_decide_kernel(const double* __r
 
 constexpr int kPfSeg = 16;  // output frames of one moving-average thread
 
-constexpr float kPfRange = 1e36f;  // a partial sum at or above it (or not a number) sends the segment to FP64
+// A partial sum at or above kPfRange (or not a number), or a window sum so small that the
+// errors of its products would underflow, sends the segment to FP64.
+constexpr float kPfRange = 1e36f, kPfTiny = 1e-25f;
 
-// (h, l) += x, the rounding error of h + x kept in l (Knuth's TwoSum)
-__device__ __forceinline__ void pf_add(float& h, float& l, float x) {
-  const float s = __fadd_rn(h, x), z = __fsub_rn(s, h);
-  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(x, z)));
-  h = s;
+// s + e = a + b exactly (Knuth's TwoSum)
+__device__ __forceinline__ void pf_two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float z = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
 }
+
+// (h, l, t) += x: the rounding error of h + x goes to l, that of l to t, which leaves
+// about 2^-72 of the largest partial sum
+__device__ __forceinline__ void pf_add(float& h, float& l, float& t, float x) {
+  float e;
+  pf_two_sum(h, x, h, e);
+  pf_two_sum(l, e, l, e);
+  t = __fadd_rn(t, e);
+}
+
+// 1 / window as the sum of three floats (to about 2^-72)
+struct PfInv {
+  float h, l, t;
+};
 
 // Output frames j0 .. j1-1 of pixel p with FP64 sums.
 template <bool HP>
@@ -173,15 +191,13 @@ __device__ __noinline__ void pf_segment64(const float* X, int64_t m, const int* 
 template <bool HP>
 __global__ void __launch_bounds__(kPfThreads) pf_average_kernel(const float* __restrict__ X, int64_t m, int T,
                                                                 const int* __restrict__ kept,
-                                                                const int* __restrict__ count, int window,
+                                                                const int* __restrict__ count, int window, PfInv iw,
                                                                 float* __restrict__ Y) {
   extern __shared__ int pf_kept[];
   for (int i = threadIdx.x; i < T; i += blockDim.x) pf_kept[i] = kept[i];
   __syncthreads();
   const int n = count[1];
   if (n <= 0) return;
-  const double inv_w = 1.0 / (double)window;
-  const float ih = (float)inv_w, il = (float)(inv_w - (double)ih);
   const int h = (window - 1) / 2;
   const int64_t nseg = (n + kPfSeg - 1) / kPfSeg;
   for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < nseg * m;
@@ -189,31 +205,39 @@ __global__ void __launch_bounds__(kPfThreads) pf_average_kernel(const float* __r
     const int64_t p = it % m;
     const int j0 = (int)(it / m) * kPfSeg;
     const int j1 = (j0 + kPfSeg < n) ? j0 + kPfSeg : n;
-    float sh = 0.f, sl = 0.f;
+    float sh = 0.f, sl = 0.f, st = 0.f;
     bool wide = false;
 #pragma unroll 4
     for (int i = 0; i < window; ++i) {
-      pf_add(sh, sl, X[(int64_t)pf_kept[j0 + i] * m + p]);
+      pf_add(sh, sl, st, X[(int64_t)pf_kept[j0 + i] * m + p]);
       wide |= !(fabsf(sh) < kPfRange);
     }
 #pragma unroll 4
     for (int j = j0; j < j1; ++j) {
       if (j > j0) {
-        pf_add(sh, sl, X[(int64_t)pf_kept[j + window - 1] * m + p]);
+        pf_add(sh, sl, st, X[(int64_t)pf_kept[j + window - 1] * m + p]);
         wide |= !(fabsf(sh) < kPfRange);
-        pf_add(sh, sl, -X[(int64_t)pf_kept[j - 1] * m + p]);
+        pf_add(sh, sl, st, -X[(int64_t)pf_kept[j - 1] * m + p]);
         wide |= !(fabsf(sh) < kPfRange);
       }
-      // mean = (sh + sl)(ih + il), product error included, rounded once
-      const float q = __fmul_rn(sh, ih);
-      const float e = __fadd_rn(fmaf(sh, ih, -q), fmaf(sh, il, sl * ih));
+      // mean = (a + b + c)(iw.h + iw.l + iw.t) = q + v + r, the leading products exact
+      float a, b, c, u, v, e1, e2;
+      pf_two_sum(sh, sl, a, b);
+      pf_two_sum(b, st, b, c);
+      wide |= a != 0.f && fabsf(a) < kPfTiny;
+      const float q = __fmul_rn(a, iw.h), q1 = fmaf(a, iw.h, -q);
+      const float al = __fmul_rn(a, iw.l), al1 = fmaf(a, iw.l, -al);
+      const float bh = __fmul_rn(b, iw.h), bh1 = fmaf(b, iw.h, -bh);
+      pf_two_sum(al, bh, u, e1);
+      pf_two_sum(q1, u, v, e2);
+      const float r = fmaf(a, iw.t, fmaf(b, iw.l, fmaf(c, iw.h, al1 + bh1))) + (e1 + e2);
       if (HP) {
-        const float x = X[(int64_t)pf_kept[j + h] * m + p];
-        float dh = x, dl = 0.f;
-        pf_add(dh, dl, -q);
-        Y[(int64_t)j * m + p] = __fadd_rn(dh, __fsub_rn(dl, e));
+        float d, f, d1, f1;
+        pf_two_sum(X[(int64_t)pf_kept[j + h] * m + p], -q, d, d1);
+        pf_two_sum(d, -v, f, f1);
+        Y[(int64_t)j * m + p] = __fadd_rn(f, __fsub_rn(__fadd_rn(d1, f1), r));
       } else {
-        Y[(int64_t)j * m + p] = __fadd_rn(q, e);
+        Y[(int64_t)j * m + p] = __fadd_rn(q, __fadd_rn(v, r));
       }
     }
     if (wide) pf_segment64<HP>(X, m, pf_kept, window, Y, p, j0, j1);
@@ -245,10 +269,15 @@ rpca_status prefilter_impl(const float* X, int64_t m, int32_t T, double corr_min
   const int64_t items = m * (int64_t)((T + kPfSeg - 1) / kPfSeg);  // at most this many (segment, pixel) items
   const int64_t want = (items + kPfThreads - 1) / kPfThreads;
   const int grid = (int)(want < (int64_t)sms * 8 ? want : (int64_t)sms * 8);
+  const double inv = 1.0 / (double)window, rest = fma(-(double)window, inv, 1.0) * inv;  // inv + rest: 1 / window to 2^-106
+  PfInv iw;
+  iw.h = (float)inv;
+  iw.l = (float)(inv - (double)iw.h);
+  iw.t = (float)((inv - (double)iw.h - (double)iw.l) + rest);
   if (high_pass)
-    pf_average_kernel<true><<<grid, kPfThreads, sizeof(int) * (size_t)T, s>>>(X, m, T, kept, count, window, Y);
+    pf_average_kernel<true><<<grid, kPfThreads, sizeof(int) * (size_t)T, s>>>(X, m, T, kept, count, window, iw, Y);
   else
-    pf_average_kernel<false><<<grid, kPfThreads, sizeof(int) * (size_t)T, s>>>(X, m, T, kept, count, window, Y);
+    pf_average_kernel<false><<<grid, kPfThreads, sizeof(int) * (size_t)T, s>>>(X, m, T, kept, count, window, iw, Y);
   return cudaGetLastError() == cudaSuccess ? RPCA_OK : RPCA_ERR_CUDA;
 }
 
