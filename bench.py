@@ -95,15 +95,21 @@ def ncu_batch_traffic(kernel_src_hash: str, iters, entry: str = "batch_kernel"):
     return sum(per_window * (1 + 5 * it + 5) / (1 + 5 * it0 + 5) for it in iters)
 
 
-TILED_HEADERS = ("rpca_wide.cuh", "rpca_wide_tc.cuh")
+TILED_HEADERS = ("rpca_wide.cuh", "rpca_wide_tc.cuh", "rpca_eig_wide.cuh")
+
+
+def prefilter_fp64_ops(m: int, T: int) -> int:
+    """FP64 pipe operations of a pre-filter call: its statistics, 7 per element
+    (two FP32->FP64 conversions, two shifts, the sum, two FMAs).  The averages
+    run on the FP32 pipe."""
+    return 7 * m * T
 
 
 def kernel_source_hash() -> str:
     """Hash of the device code of the register-resident (narrow) solver, which
     the committed ncu summaries cover: its kernel bodies live in the csrc/*.cuh
-    headers other than the tiled path's rpca_wide.cuh and rpca_wide_tc.cuh (the
-    tiled batch kernel's rpca_batch_wide.cu and host-only sources do not enter
-    it either)."""
+    headers other than the tiled path's own, TILED_HEADERS (the tiled batch
+    kernel's rpca_batch_wide.cu and host-only sources do not enter it either)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2506_10257_gb300", "csrc")
     for fn in sorted(os.listdir(csrc)):
@@ -642,11 +648,10 @@ def run_prefilter(args):
         ms.append(e0.elapsed_time(e1))
     ms_mean = statistics.mean(ms)
     alg = 4 * m * (T + K + n)                    # read X (statistics), read the kept frames, write the outputs
-    aop = 8 if hp else 6
     line = {
         "metric": "pre-filters/s", "value": world * 1000.0 / ms_mean, "unit": "pre-filters/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_mean, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "f64 accumulation, f32 data",
+        "scaling": "weak", "vs_baseline": None, "dtype": "f64 statistics, three-float window sums, f32 data",
         "data": "synthetic (seeded microbubble window, three frames displaced)",
         "config": {"workload": f"frame pre-filter, {ny}x{nx} px x {T} frames (corr >= 0.8, {wdw}-frame "
                                + ("high-pass)" if hp else "average)"),
@@ -655,14 +660,10 @@ def run_prefilter(args):
                            + "; stream-ordered)",
                    "l2": "flushed before every call (256 MB write, outside the events)"},
         "kept_frames": K, "output_frames": n,
-        # FP64 pipe operations of a call: statistics 7 per element (two FP32->FP64
-        # conversions, two shifts, the sum, two FMAs), averages 6 per output
-        # (two conversions, two adds, the scale, the FP32 conversion; the high-pass
-        # two more: the centre frame's conversion and the subtraction); peak: the
-        # measured FP64 FMA rate of 1.89 per SM per clock x 152 SMs x 2.07 GHz
-        "roofline": {"bound": "alu (FP64 pipe)", "achieved": (7 * T * m + aop * n * m) / (ms_mean * 1e-3) / 1e9,
+        # peak: the measured FP64 FMA rate of 1.89 per SM per clock x 152 SMs x 2.07 GHz
+        "roofline": {"bound": "alu (FP64 pipe)", "achieved": prefilter_fp64_ops(m, T) / (ms_mean * 1e-3) / 1e9,
                      "peak": 152 * 1.89 * 2.07, "unit": "GFLOP/s (FP64 pipe ops)",
-                     "frac": (7 * T * m + aop * n * m) / (ms_mean * 1e-3) / 1e9 / (152 * 1.89 * 2.07),
+                     "frac": prefilter_fp64_ops(m, T) / (ms_mean * 1e-3) / 1e9 / (152 * 1.89 * 2.07),
                      "traffic": None, "hbm_achieved_gbs": alg / (ms_mean * 1e-3) / 1e9,
                      "hbm_peak_gbs": measured_peaks()[0], "algorithmic_bytes_per_launch": alg},
         "gpu_launches": 3 * args.steps,
