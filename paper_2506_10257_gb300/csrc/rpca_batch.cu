@@ -420,7 +420,7 @@ rpca_status rpca_batch_create(const rpca_params* params, int32_t n, rpca_batch_t
     size_t need = 0;
     for (int i = 0; i < n; ++i) {
       const int Tr = params[i].dtype == RPCA_C64 ? 2 * params[i].T : params[i].T;
-      need = std::max({need, tile_pass_smem(Tr, wide_rp(Tr, cplx), cplx), eig_wide_smem(Tr)});
+      need = std::max({need, tile_pass_smem(Tr, wide_rp(Tr, cplx), cplx), Tr <= kMaxT ? sizeof(Eig64Smem) : eig_wide_smem(Tr)});
     }
     if (need > room) {
       delete b;

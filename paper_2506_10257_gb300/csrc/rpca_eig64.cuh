@@ -1,6 +1,9 @@
 // rpca_eig64.cuh -- the narrow eigen-step (T <= 32): from the reduced Gram of
 // the rotated Z to Wbar and the next basis, to well beyond FP32 (included inside
-// namespace rpca by rpca_kernels.cuh).  One CTA of kEigThreads threads.
+// namespace rpca by rpca_kernels.cuh).  One CTA of kEigThreads threads, or the
+// threads of a batch's CTA.  Windows of the tiled path with at most 32 real
+// columns (complex ones of up to 16 frames, short ones in a batch with long
+// ones) take it too (b.wide says where G, V and Wbar lie).
 //
 // GB300 runs FP64 at about 1/64 of its FP32 rate, so FP64 Jacobi sweeps bound
 // this step (262144 x 20: 105 us, of which 83 us sweeps; x 29: 310 us).  Here the
@@ -67,7 +70,8 @@ __device__ __forceinline__ void fast_two_sum(float s, float c, float& h, float& 
   l = __fsub_rn(c, __fsub_rn(h, s));
 }
 
-static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond,
+// Returns whether the solve goes on (Wbar and V are written).
+static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphConditionalHandle h, int use_cond,
                                                unsigned char* dsm) {
   Eig64Smem& S = *reinterpret_cast<Eig64Smem*>(dsm);
   constexpr int LD = Eig64Smem::LD;
@@ -81,6 +85,10 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
   const int JL = jac_ld(T), nb = jac_blocks(T);
   const unsigned long long t0 = gtimer();
   const bool init = (flags & EF_INIT) != 0;
+  float* Vg = b.wide ? b.Vw : b.eig->V32;
+  float* Wg = b.wide ? b.Ww : b.eig->Wbar;
+  const double* Gg = b.wide ? b.Gw : b.red->G;
+  const int ldg = b.wide ? T : kMaxT;
 
   // T x T arrays: row = warp, warp + 8, ..., column = lane.  Upper triangles: entries
   // (ep, eq) of this thread (at most ceil(528 / 256) = 3).
@@ -100,13 +108,13 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int r = warp + u * nwarps;
-    v0[u] = init ? (r == lane ? 1.f : 0.f) : (r < T && lane < T) ? __ldcg(&b.eig->V32[r * kMaxT + lane]) : 0.f;
+    v0[u] = init ? (r == lane ? 1.f : 0.f) : (r < T && lane < T) ? __ldcg(&Vg[r * ldg + lane]) : 0.f;
   }
   const bool go = eig_control(b, flags, h, use_cond, &sCtl, [&](int i0, int n) {
     if (b.finalize) {
       for (int i = i0; i < TT; i += n) {
         const int r = i / T, c = i % T;
-        const double x = __ldcg(&b.red->G[r * kMaxT + c]);
+        const double x = __ldcg(&Gg[r * ldg + c]);
         const float xh = (float)x;
         S.Hh[r * LD + c] = xh;
         S.Hl[r * LD + c] = (float)(x - (double)xh);
@@ -120,7 +128,7 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
   });
   if (!go) {
     if (tid == nthr - 1) eig_control_tail(b, &sCtl);
-    return;
+    return false;
   }
 
   // ---- the Gram scaled by a power of four to about 1; the basis ----
@@ -338,7 +346,7 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
     const float p = __fmul_rn(ph, gh);
     const float e = fmaf(ph, gh, -p) + fmaf(ph, S.gl[c], S.Vl[r * LD + c] * gh);
     fast_two_sum(p, e + s, S.Nh[r * LD + c], S.Nl[r * LD + c]);
-    b.eig->V32[r * kMaxT + c] = ph;  // (normalised: the pair rounded to FP32)
+    Vg[r * ldg + c] = ph;  // (normalised: the pair rounded to FP32)
   }
   const int rank = __syncthreads_count(tid < T && S.keep[tid]);
 #pragma unroll
@@ -353,10 +361,10 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
       e = fmaf(kh, S.Vl[q * LD + k], fmaf(S.Nl[p * LD + k], ph, e));
     }
     const float w = -(s + e);
-    b.eig->Wbar[p * kMaxT + q] = w;
-    b.eig->Wbar[q * kMaxT + p] = w;
+    Wg[p * ldg + q] = w;
+    Wg[q * ldg + p] = w;
   }
-  if (tid < T) b.eig->evals[tid] = S.d[tid] / (double)scale;
+  if (tid < T) (b.wide ? b.evw : b.eig->evals)[tid] = S.d[tid] / (double)scale;
   if (tid == 0) {
     ctrl->rank = rank;
     ctrl->sweeps = sweeps;
@@ -371,6 +379,7 @@ static __device__ __noinline__ void eig64_body(Bufs b, int flags, cudaGraphCondi
     ctrl->eig_rounds += sweeps * (nb - 1);
     set_cond(h, use_cond, 1u);
   }
+  return true;
 }
 
 static __global__ void __launch_bounds__(kEigThreads) eig64_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,

@@ -559,7 +559,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   if (lane == 0) S.perm[warp] = kept;
   if (b.wtc) {
     eig_sync(nr);  // Ww and Vw written by every rank
-    wtc_images(b, M(ES_VT), ld, rank, nr);
+    wtc_images(b, M(ES_VT), ld, 1, rank, nr);
   } else {
     __syncthreads();
   }

@@ -38,7 +38,7 @@ WideKernels make_wide() {
   return k;
 }
 
-size_t wide_eig_scr_bytes(int T) { return eig_scr_bytes(T); }
+size_t wide_eig_scr_bytes(int T) { return T <= kMaxT ? 1 : eig_scr_bytes(T); }
 
 size_t wide_tc_img_bytes(int T, int precision) {
   const int TP = wtc_tp(T);
@@ -69,16 +69,23 @@ bool wide_kernels(int T, bool cplx, bool force, int64_t m, int sms, WideKernels*
     default: *out = make_wide<256, 64, true>(); break;
   }
   out->pass_smem = tile_pass_smem(T, RP, cplx);
-  // the sweeps' columns, or one rank's operands of a product, as far as they fit
-  const size_t ops = 2 * sizeof(float) * (size_t)T * (eig_ld(T) + (eig_ld(T) / 4 + kEigWRanks - 1) / kEigWRanks * 4);
-  out->eig_smem = eig_wide_smem(T);
-  if (ops > out->eig_smem) out->eig_smem = ops < kEigWMaxSmem ? ops : (out->eig_smem > kEigWMaxSmem ? out->eig_smem : kEigWMaxSmem);
   // The kernels are shared by plans of other frame counts, which may have been made before and launch with their own
   // size: the limits are those of the largest one, whatever this plan needs.
-  static_assert(eig_wide_smem(kMaxTW) <= kEigWMaxSmem, "the sweeps of the longest columns fit");
   const int pass_max = (int)tile_pass_smem(std::min(tile_tp(T, cplx), kMaxTW), RP, cplx);
-  if (cudaFuncSetAttribute(out->eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEigWMaxSmem) != cudaSuccess)
-    return false;
+  size_t eig_max;
+  if (T <= kMaxT) {
+    out->eig = (void*)eig_small_kernel;
+    out->eig_threads = kEigThreads;
+    out->eig_ctas = 1;
+    out->eig_smem = eig_max = sizeof(Eig64Smem);
+  } else {
+    // the sweeps' columns, or one rank's operands of a product, as far as they fit
+    const size_t ops = 2 * sizeof(float) * (size_t)T * (eig_ld(T) + (eig_ld(T) / 4 + kEigWRanks - 1) / kEigWRanks * 4);
+    static_assert(eig_wide_smem(kMaxTW) <= kEigWMaxSmem, "the sweeps of the longest columns fit");
+    out->eig_smem = std::max(eig_wide_smem(T), std::min(ops, kEigWMaxSmem));
+    eig_max = kEigWMaxSmem;
+  }
+  if (cudaFuncSetAttribute(out->eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eig_max) != cudaSuccess) return false;
   for (int i = 0; i < 4; ++i)
     if (cudaFuncSetAttribute(out->pass[i], cudaFuncAttributeMaxDynamicSharedMemorySize, pass_max) != cudaSuccess)
       return false;

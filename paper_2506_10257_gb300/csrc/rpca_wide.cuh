@@ -651,19 +651,32 @@ __global__ void __launch_bounds__(kWideThreads, tile_blocks_per_sm(TP, CPLX)) pa
 
 // The B operand images of the tiled tensor-core pass (b.wtc), written by the
 // eigen-step once Ww and Vw are final.
-__device__ __forceinline__ void wtc_images(const Bufs& b, const float* vt, int ldv, int rank, int nr) {
+__device__ __forceinline__ void wtc_images(const Bufs& b, const float* v, int sn, int sk, int rank, int nr) {
   const int TP = wtc_tp(b.T);
   if (b.wtc == 1) {
-    if (TP == 64) wtc_write_images<64, false>(b, vt, ldv, rank, nr);
-    else if (TP == 96) wtc_write_images<96, false>(b, vt, ldv, rank, nr);
-    else if (TP == 128) wtc_write_images<128, false>(b, vt, ldv, rank, nr);
+    if (TP == 64) wtc_write_images<64, false>(b, v, sn, sk, rank, nr);
+    else if (TP == 96) wtc_write_images<96, false>(b, v, sn, sk, rank, nr);
+    else if (TP == 128) wtc_write_images<128, false>(b, v, sn, sk, rank, nr);
   } else if (b.wtc == 2) {
-    if (TP == 64) wtc_write_images<64, true>(b, vt, ldv, rank, nr);
-    else if (TP == 96) wtc_write_images<96, true>(b, vt, ldv, rank, nr);
-    else if (TP == 128) wtc_write_images<128, true>(b, vt, ldv, rank, nr);
+    if (TP == 64) wtc_write_images<64, true>(b, v, sn, sk, rank, nr);
+    else if (TP == 96) wtc_write_images<96, true>(b, v, sn, sk, rank, nr);
+    else if (TP == 128) wtc_write_images<128, true>(b, v, sn, sk, rank, nr);
   }
 }
 
 #include "rpca_eig_wide.cuh"
+
+// The eigen-step of a plan of at most kMaxT real columns on the tiled path: the
+// narrow one on one CTA, then the operand images.  The cluster's products and
+// barriers cost more there than the whole narrow step: measured, a 4-frame
+// complex 64 x 64 window 1.43 -> 0.75 ms a solve.
+static __global__ void __launch_bounds__(kEigThreads) eig_small_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,
+                                                                       int use_cond, int) {
+  extern __shared__ __align__(16) unsigned char eigs_smem[];
+  if (eig64_body(b, flags, h, use_cond, eigs_smem) && b.wtc) {
+    __syncthreads();  // Ww and Vw written
+    wtc_images(b, b.Vw, 1, b.T, 0, 1);
+  }
+}
 
 }  // namespace rpca

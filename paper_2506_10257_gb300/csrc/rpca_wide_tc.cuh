@@ -113,18 +113,19 @@ __device__ __forceinline__ void tc_store1(unsigned char* hi, unsigned char* lo, 
 // The B operand images of Wbar and V for the pass (called by the eigen-step
 // CTA after it has written Ww and Vw): image [m][c] holds rows n < TP and
 // frames k of chunk c of B[n][k] = M[k][n] (M = Wbar or V), zero outside T.
+// V's entry of frame k and column n is v[n * sn + k * sk].
 template <int TP, bool BF16>
-__device__ void wtc_write_images(const Bufs& b, const float* vt, int ldv, int rank, int nr) {
+__device__ void wtc_write_images(const Bufs& b, const float* v, int sn, int sk, int rank, int nr) {
   using SH = WtcShape<TP, BF16>;
   const int T = b.T;
   for (int i = threadIdx.x + rank * blockDim.x; i < 2 * TP * TP; i += nr * blockDim.x) {
     const int mat = i / (TP * TP), e = i % (TP * TP);
     const int n = e / TP, k = e % TP;
-    // (row n of V^T, and of Wbar, which is symmetric: consecutive k)
-    const float v = (n < T && k < T) ? __ldcg(mat ? &vt[n * ldv + k] : &b.Ww[n * T + k]) : 0.f;
+    // (Wbar is symmetric: row n has consecutive k)
+    const float x = (n < T && k < T) ? __ldcg(mat ? &v[n * sn + k * sk] : &b.Ww[n * T + k]) : 0.f;
     const int c = k / kWtcKCh;
     unsigned char* hi = b.wtc_img + ((size_t)(mat * SH::NCH + c) * 2) * SH::B_BYTES;
-    tc_store1<BF16>(hi, hi + SH::B_BYTES, SH::off(n, k % kWtcKCh), v);
+    tc_store1<BF16>(hi, hi + SH::B_BYTES, SH::off(n, k % kWtcKCh), x);
   }
 }
 
