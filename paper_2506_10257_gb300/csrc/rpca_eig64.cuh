@@ -20,11 +20,11 @@
 //                                 E_pq = Gp_pq - max(d_p, d_q) Omega_pq.
 // Wbar = f(Z^T Z) with f(sigma^2) = min(1, tau / sigma) is then
 //   I - P (diag(1 - g) - F o E) P^T,  F the divided differences of f
-// (g_divided_difference), right to second order in E and Omega; only the vectors
+// (g_divided_difference), right to first order in E and Omega; only the vectors
 // with sigma > tau enter it, so the others need not be separated from one another
-// and the sweeps stop once what is neglected on the former is below the result's
-// FP32 rounding.  A step that finds more left there runs another round of sweeps
-// on diag(d) + E.  sigma, the sigma > tau decision, g and mu are FP64.  Measured on
+// and the sweeps stop once what is neglected is about the result's FP32 rounding,
+// the kink of f at tau included (rpca_eig_rule.cuh).  A step that finds more left
+// runs another round of sweeps on diag(d) + E.  sigma, the sigma > tau decision, g and mu are FP64.  Measured on
 // the windows above: 25 us (load 3, factor and sweeps 13, products and decisions 10)
 // and 44 us, at the same errors of L and S against 64 bits (1.0e-7 and 2.3e-7).
 #pragma once
@@ -33,10 +33,6 @@ constexpr int kEigThreads = 256;   // threads of the eigen-step CTA
 constexpr int kEigPasses = 3;      // rounds of sweeps one eigen-step may take
 constexpr float kEigStop = 3e-3f;  // largest cosine a sweep may meet and be the last
 constexpr float kEigInitStop = 1e-5f;  // ... of the first eigen-step, whose largest eigenvalue sets mu
-constexpr float kEigMaxOff = 4e-4f;    // largest |E_pq| corrected to first order, relative to sigma_p sigma_q where
-                                       // both enter Wbar, else to the larger sigma^2: what is neglected, 3/8 of
-                                       // its square, is FP32's rounding
-constexpr float kEigMaxOm = 2.4e-4f;    // largest |Omega_pq| (its square is neglected)
 constexpr float kEigNear = 0.25f;       // a sweep's cosines count where the longer column's sigma^2 / tau^2 is above this
 
 struct Eig64Smem {
@@ -182,9 +178,9 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     __syncthreads();
     jac_cholesky<1>(S.W, JL, T, S.diag, S.piv);
     // the pairs that Wbar depends on: those with a singular value near or above tau
-    // (the first step's tau comes from its eigenvalues, a further pass wants them all)
+    // (the first step wants them all: its tau comes from its eigenvalues)
     const float taus = (float)(sTau * root);
-    const float lim = init || pass ? 0.f : fminf(kEigNear * taus * taus, 0.5f * S.diag[0]);
+    const float lim = init ? 0.f : fminf(kEigNear * taus * taus, 0.5f * S.diag[0]);
     const float stop = init ? kEigInitStop : kEigStop;
     const int cap = (init || (flags & EF_FULL)) ? 16 : 8;
     sweeps += jac_r2(T) == 1 ? jac_sweeps<1>(S.W, JL, nb, S.nrm, S.smax, stop, lim, cap)
@@ -295,9 +291,7 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
       S.B[q * LD + p] = bv;
     }
     __syncthreads();
-    // ---- P = Vn (I - C); whether E is small enough.  Pairs of two singular values
-    //      below tau do not enter Wbar, unless what the sweeps left between them
-    //      could hide an eigenvalue above tau^2 (Gershgorin's bound of the row) ----
+    // ---- P = Vn (I - C); whether E is small enough (rpca_eig_rule.cuh) ----
 #pragma unroll 1
     for (int r = warp; r < T; r += nwarps) {
       const int c = lane < T ? lane : 0;
@@ -305,15 +299,19 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
 #pragma unroll 4
       for (int k = 0; k < T; ++k) s = fmaf(S.Nh[r * LD + k], S.C[k * LD + c], s);
       const float sr = S.sig[r], sc = S.sig[c], ev = fabsf(S.E[r * LD + c]);
-      const bool kept = S.keep[r] || S.keep[c], both = S.keep[r] && S.keep[c];
-      const float hi = fmaxf(sr, sc);
-      const bool off = lane < T && r != c && (ev > kEigMaxOff * hi * (both ? fminf(sr, sc) : hi) ||
-                                           fabsf(S.Om[min(r, c) * LD + max(r, c)]) > kEigMaxOm);
-      if (off && kept) more = 1;
-      float hid = off && !kept ? ev : 0.f;
+      const float hi = fmaxf(sr, sc), lo = fminf(sr, sc), om = fabsf(S.Om[min(r, c) * LD + max(r, c)]);
+      const int kept = S.keep[r] + S.keep[c];
+      const bool pair = lane < T && r != c;
+      if (pair && kept && eig_pair_off(ev, om, hi, lo, kept)) more = 1;
+      auto row_off = [&](float shift) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) hid += __shfl_xor_sync(0xffffffffu, hid, o);
-      if (hid > 0.f && !S.keep[r] && fmaf(sr, sr, hid) > tauf * tauf) more = 1;
+        for (int o = 16; o > 0; o >>= 1) shift += __shfl_xor_sync(0xffffffffu, shift, o);
+        return eig_row_off(S.keep[r], sr, shift, tauf);
+      };
+      // (a bound without divisions first: few rows lie near tau)
+      if (row_off(pair && kept != 1 ? eig_pair_most(ev, om, hi) : 0.f) &&
+          row_off(pair && kept != 1 ? eig_pair_shift(ev, om, hi, lo) : 0.f))
+        more = 1;
       if (lane < T) fast_two_sum(S.Nh[r * LD + c], S.Nl[r * LD + c] - s, S.Vh[r * LD + c], S.Vl[r * LD + c]);
     }
     more = __syncthreads_or(more);

@@ -329,7 +329,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
         for (int i = tid; i < TT; i += nthr) M(ES_VT)[i / T * ld + i % T] = i / T == i % T ? 1.f : 0.f;
       __syncthreads();
       const float taus = (float)(tau * (double)rootf);
-      const float lim = init || pass ? 0.f : fminf(kEigNear * taus * taus, 0.5f * S.diag[0]);
+      const float lim = init ? 0.f : fminf(kEigNear * taus * taus, 0.5f * S.diag[0]);
       sweeps += eig_wide_factor(sm, T, S, init ? kEigInitStop : kEigWStop, lim,
                                 (init || (flags & EF_FULL)) ? 16 : 8);
       // D = U - I from the normalised columns
@@ -455,10 +455,10 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       S.g1l[i] = (float)(g1 - (double)(float)g1);
     }
     __syncthreads();
-    // ---- C, -F o E, E, and whether E and Omega are small enough ----
+    // ---- C, -F o E, E, and whether E (beyond its FP32 rounding) and Omega are small enough ----
     int more = 0;
     for (int p = rank + nr * warp; p < T; p += nr * nwarps) {
-      float hid = 0.f;
+      float most = 0.f;
       const float sp = S.sig[p], dp = (float)S.d[p];
       const int kp = S.keep[p];
       for (int q = lane; q < T; q += 32) {
@@ -476,14 +476,26 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
         M(ES_C)[p * ld + q] = pbig ? om : 0.f;
         M(ES_B)[p * ld + q] = -g_divided_difference(hi, lo, tauf) * ev;
         M(ES_E)[p * ld + q] = ev;
-        const bool off =
-            fabsf(ev) > kEigMaxOff * hi * (kp && S.keep[q] ? lo : hi) + kEigNoise * dm || fabsf(om) > kEigMaxOm;
-        if (off && (kp || S.keep[q])) more = 1;
-        if (off && !kp && !S.keep[q]) hid += fabsf(ev);
+        const float e = fmaxf(fabsf(ev) - kEigNoise * dm, 0.f);
+        const int kept = kp + S.keep[q];
+        if (kept && eig_pair_off(e, fabsf(om), hi, lo, kept)) more = 1;
+        if (kept != 1) most += eig_pair_most(e, fabsf(om), hi);
       }
+      auto row_off = [&](float shift) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) hid += __shfl_xor_sync(0xffffffffu, hid, o);
-      if (hid > 0.f && !kp && fmaf(sp, sp, hid) > tauf * tauf) more = 1;
+        for (int o = 16; o > 0; o >>= 1) shift += __shfl_xor_sync(0xffffffffu, shift, o);
+        return eig_row_off(kp, sp, shift, tauf);
+      };
+      if (row_off(most)) {  // (a bound without divisions: few rows lie near tau)
+        float shift = 0.f;
+        for (int q = lane; q < T; q += 32) {
+          if (q == p || S.keep[q] != kp) continue;
+          const float sq = S.sig[q], dm = fmaxf(dp, (float)S.d[q]);
+          const float e = fmaxf(fabsf(M(ES_E)[p * ld + q]) - kEigNoise * dm, 0.f);  // (this lane's own store)
+          shift += eig_pair_shift(e, fabsf(__ldcg(&M(ES_OM)[p * ld + q])), fmaxf(sp, sq), fminf(sp, sq));
+        }
+        if (row_off(shift)) more = 1;
+      }
     }
     more = __syncthreads_or(more);
     if (more && tid == 0) atomicOr(&gflag[1 + pass], 1);

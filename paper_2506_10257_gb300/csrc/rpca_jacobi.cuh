@@ -23,6 +23,8 @@
 // inner product - three shuffles - square root - rotation.
 #pragma once
 
+#include "rpca_eig_rule.cuh"
+
 // Row pairs (float2) a lane holds per column: the frame count rounded up to a
 // multiple of 16 rows, in the sizes below.
 __host__ __device__ constexpr int jac_r2(int T) {
