@@ -187,6 +187,14 @@ rpca_status rpca_plan_result(rpca_plan_t plan, rpca_result* out);
  * untouched.  Implementation instrumentation: the paper has no counterpart. */
 rpca_status rpca_plan_timings(rpca_plan_t plan, double* out, int32_t n);
 
+/* How the eigen-steps of the last solve went (after synchronising its stream):
+ * *further counts the rounds of sweeps that steps took beyond their first,
+ * *unfinished the steps that used up their rounds with the eigenvectors still
+ * further from orthogonal than their correction is exact for (Wbar is then
+ * less accurate than FP32's rounding; the residual test still holds for what
+ * the solve returns).  RPCA_ERR_ARG for a null pointer. */
+rpca_status rpca_plan_eig_rounds(rpca_plan_t plan, int32_t* further, int32_t* unfinished);
+
 void rpca_plan_destroy(rpca_plan_t plan);
 
 const char* rpca_status_str(int32_t status);

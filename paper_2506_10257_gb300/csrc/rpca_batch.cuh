@@ -160,6 +160,8 @@ __device__ __forceinline__ void reset_window(WinDesc& wd) {
   for (int i = 0; i < 4; ++i) c->eig_phase_ns[i] = 0ull;
   for (int i = 0; i < 3; ++i) c->pass_phase_ns[i] = 0ull;
   c->eig_rounds = 0;
+  c->eig_further = 0;
+  c->eig_unfinished = 0;
   b.red->t_start = ~0ull;
   b.red->t_end = 0ull;
   b.red->t_loop = 0ull;

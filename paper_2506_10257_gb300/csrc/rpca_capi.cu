@@ -788,6 +788,14 @@ rpca_status rpca_plan_timings(rpca_plan_t pl, double* out, int32_t n) {
   return RPCA_OK;
 }
 
+rpca_status rpca_plan_eig_rounds(rpca_plan_t pl, int32_t* further, int32_t* unfinished) {
+  if (!pl || !further || !unfinished) return RPCA_ERR_ARG;
+  CK(cudaMemcpy(pl->ctrl_host, pl->bufs.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost));
+  *further = pl->ctrl_host->eig_further;
+  *unfinished = pl->ctrl_host->eig_unfinished;
+  return RPCA_OK;
+}
+
 void rpca_plan_destroy(rpca_plan_t pl) {
   if (!pl) return;
   if (pl->stage_x) cudaFree(pl->stage_x);

@@ -79,6 +79,8 @@ struct Ctrl {
   // last CTA's partials, first-level reduction, final reduction
   unsigned long long pass_phase_ns[3];
   int eig_rounds;    // Jacobi rounds executed (summed)
+  int eig_further;   // rounds of sweeps that eigen-steps took beyond their first (summed)
+  int eig_unfinished;  // eigen-steps that took kEigPasses rounds and still found E or Omega too large
   int pad_;
 };
 

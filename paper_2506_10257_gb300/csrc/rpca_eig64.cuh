@@ -30,7 +30,7 @@
 #pragma once
 
 constexpr int kEigThreads = 256;   // threads of the eigen-step CTA
-constexpr int kEigPasses = 3;      // rounds of sweeps one eigen-step may take
+constexpr int kEigPasses = 8;      // rounds of sweeps one eigen-step may take
 constexpr float kEigStop = 3e-3f;  // largest cosine a sweep may meet and be the last
 constexpr float kEigInitStop = 1e-5f;  // ... of the first eigen-step, whose largest eigenvalue sets mu
 constexpr float kEigNear = 0.25f;       // a sweep's cosines count where the longer column's sigma^2 / tau^2 is above this
@@ -48,7 +48,7 @@ struct Eig64Smem {
   double d[kMaxT];
   float sig[kMaxT], gh[kMaxT], gl[kMaxT] /* 1 - g */, diag[kMaxT], piv[kMaxT], nrm[kMaxT];
   int perm[kMaxT], keep[kMaxT];
-  unsigned smax[2];
+  unsigned smax[2], lift;
 };
 
 // Dot2: (s, c) += a b, with the rounding errors of the product and of the sum in c.
@@ -142,14 +142,15 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     S.Nl[r * LD + lane] = 0.f;
   }
   if (tid < 2) S.smax[tid] = 0u;
+  if (tid == 0) S.lift = 0u;
   if (tid == 0) sTau = sCtl.tau;
   const double root = (double)rootf;
   __syncthreads();
   const unsigned long long t1 = gtimer();
   unsigned long long t2 = t1, t3 = t1;
-  int sweeps = 0;
+  int sweeps = 0, pass = 0, more = 0;
   const double mu_prev = init ? __ldcg(&ctrl->mu_cur) : 0.0;  // (of the plan's previous solve)
-  for (int pass = 0;; ++pass) {
+  for (;; ++pass) {
     // ---- descending order of the diagonal; Cholesky factor; one-sided Jacobi ----
     // (every warp works the order out and writes the same values)
     const float dl = lane < T ? S.Hh[lane * LD + lane] : 0.f;
@@ -163,16 +164,20 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     __syncwarp();
     auto perm = [&](int i) { return min((unsigned)S.perm[i < T ? i : 0], (unsigned)(T - 1)); };  // (in range for any values)
     const int pl = perm(lane);
+    // a further round's matrix may be indefinite: shifted by at least twice its most
+    // negative eigenvalue it has a factor, and the same eigenvectors
+    const float lift = 2.f * __uint_as_float(S.lift);
     for (int c = warp; c < 4 * nb; c += nwarps) {
       const int pc = perm(c);
-      if (lane < 16 * jac_r2(T)) S.W[c * JL + lane] = (lane < T && c <= lane) ? S.Hh[pl * LD + pc] : 0.f;
+      if (lane < 16 * jac_r2(T))
+        S.W[c * JL + lane] = (lane < T && c <= lane) ? S.Hh[pl * LD + pc] + (c == lane ? lift : 0.f) : 0.f;
       if (c < T && lane < T) {
         const float gh = S.Hh[pc * LD + pl];
         S.Gh[c * LD + lane] = gh;
         S.Gl[c * LD + lane] = S.Hl[pc * LD + pl];
         S.Vh[c * LD + lane] = S.Nh[c * LD + pl];
         S.Vl[c * LD + lane] = S.Nl[c * LD + pl];
-        if (c == lane) S.diag[c] = gh;
+        if (c == lane) S.diag[c] = gh + lift;
       }
     }
     __syncthreads();
@@ -194,6 +199,7 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     }
     if (tid < 2) S.smax[tid] = 0u;
     __syncthreads();
+    if (tid == 0) S.lift = 0u;
     t2 = gtimer();
     // ---- Vn = V U, H = G U ----
 #pragma unroll 1
@@ -266,7 +272,7 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     __syncthreads();
     // ---- E, C and -F o E ----
     const float tauf = (float)(sTau * root);
-    int more = 0;
+    more = 0;
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const int p = ep[u], q = eq[u];
@@ -316,11 +322,17 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     }
     more = __syncthreads_or(more);
     if (!more || pass + 1 == kEigPasses) break;
-    // another round on diag(d) + E in the basis P
+    // another round on diag(d) + E in the basis P; how far below zero its eigenvalues may
+    // lie (the row bound of the stopping rule)
 #pragma unroll 1
     for (int r = warp; r < T; r += nwarps) {
-      if (lane >= T) break;
-      const int c = lane;
+      const int c = lane < T ? lane : 0;
+      const float dr = (float)S.d[r], dc = (float)S.d[c];
+      float below = lane >= T ? 0.f : r == c ? -dr : eig_shift(fabsf(S.E[r * LD + c]), fabsf(dr - dc));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+      if (lane == 0 && below > 0.f) atomicMax(&S.lift, __float_as_uint(below));
+      if (lane >= T) continue;
       const double x = r == c ? S.d[r] : (double)S.E[r * LD + c];
       const float xh = (float)x;
       S.Hh[r * LD + c] = xh;
@@ -375,6 +387,8 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
     ctrl->eig_phase_ns[2] += t3 - t2;
     ctrl->eig_phase_ns[3] += t4 - t3;
     ctrl->eig_rounds += sweeps * (nb - 1);
+    ctrl->eig_further += pass;
+    ctrl->eig_unfinished += more ? 1 : 0;
     set_cond(h, use_cond, 1u);
   }
   return true;

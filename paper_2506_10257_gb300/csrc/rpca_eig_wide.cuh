@@ -36,6 +36,7 @@ __host__ __device__ constexpr size_t eig_scr_bytes(int T) {
 }
 
 constexpr int kEigWThreads = 512;   // 128 registers a thread: the longest columns of a sweep fit
+static_assert(1 + kEigPasses <= 15, "the flags of a step");
 constexpr int kEigWRanks = 8;       // CTAs of a plan's eigen-step
 constexpr float kEigWStop = 1e-3f;   // largest cosine of a last sweep: 3e-3, as in the narrow step, left one step in
                                     // four of 132 frames short, and a second round costs more than the extra sweeps
@@ -54,7 +55,7 @@ struct EigWideSh {
   double d[kMaxTW];
   float sig[kMaxTW], g1[kMaxTW], g1l[kMaxTW], diag[kMaxTW], piv[kMaxTW], nrm[kMaxTW];
   int perm[kMaxTW], keep[kMaxTW];
-  unsigned smax[2];
+  unsigned smax[2], lift;
   EigCtl ctl;
 };
 
@@ -238,7 +239,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   const size_t msz = (size_t)ld * ld;
   auto M = [&](int i) { return b.eig_scr + i * msz; };
   int* iscr = reinterpret_cast<int*>(b.eig_scr + ES_COUNT * msz);  // perm[kMaxTW], then flags
-  int* gflag = iscr + kMaxTW;  // [0] go on, [1 + pass] another pass wanted, [8] scale exponent
+  int* gflag = iscr + kMaxTW;  // [0] go on, [1 + pass] another pass wanted, [15] scale exponent
   const bool init = (flags & EF_INIT) != 0;
   const unsigned long long t0 = gtimer();
 
@@ -272,11 +273,12 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   const float* src = G;            // this pass's Gram
   const float* vt = M(ES_VT);      // the basis, transposed
   float scale = 1.f, rootf = 1.f;
-  int sweeps = 0;
+  int sweeps = 0, pass = 0;
+  bool unfinished = false;
   double tau = init ? 0.0 : __ldcg(&ctrl->inv_cur);
   const double mu_prev = init ? __ldcg(&ctrl->mu_cur) : 0.0;  // (of the plan's previous solve)
   float tauf = 0.f;
-  for (int pass = 0;; ++pass) {
+  for (;; ++pass) {
     if (rank == 0) {
       // ---- descending order of the diagonal, scaling, factor, sweeps ----
       for (int i = tid; i < T; i += nthr) {
@@ -284,14 +286,27 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
         S.perm[i] = i;
       }
       if (tid < 2) S.smax[tid] = 0u;
+      if (tid == 0) S.lift = 0u;
       __syncthreads();
-      if (pass == 0) {
+      if (pass > 0) {
+        // a further round's matrix may be indefinite: shifted by at least twice its most
+        // negative eigenvalue (the row bound of the stopping rule) it has a factor, and the
+        // same eigenvectors
+        for (int p = warp; p < T; p += nwarps) {
+          float below = 0.f;
+          for (int q = lane; q < T; q += 32)
+            below += q == p ? -S.diag[p] : eig_shift(fabsf(__ldcg(&src[p * ld + q])), fabsf(S.diag[p] - S.diag[q]));
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+          if (lane == 0 && below > 0.f) atomicMax(&S.lift, __float_as_uint(below));
+        }
+      } else {
         float mx = 0.f;
         for (int i = lane; i < T; i += 32) mx = fmaxf(mx, S.diag[i]);
         const int pw = even_exponent(mx);
         scale = exp2i(-pw);
         rootf = exp2i(-pw / 2);
-        if (tid == 0) gflag[8] = pw;
+        if (tid == 0) gflag[15] = pw;
       }
       int pos = 0;
       if (tid < T) {
@@ -305,7 +320,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       __syncthreads();
       if (tid < T) S.perm[pos] = tid;  // (in range whatever the values are)
       __syncthreads();
-      const float sc = pass == 0 ? scale : 1.f;
+      const float sc = pass == 0 ? scale : 1.f, lift = 2.f * __uint_as_float(S.lift);
       const int LD = jac_ld(T), rows = 16 * jac_r2(T);
       for (int c = warp; c < 4 * jac_blocks(T); c += nwarps) {
         const int pc = c < T ? S.perm[c] : 0;
@@ -315,11 +330,11 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
             v = __ldcg(&src[pc * ld + S.perm[r]]) * sc;
             M(ES_GS)[c * ld + r] = v;
           }
-          sm[c * LD + r] = c <= r ? v : 0.f;
+          sm[c * LD + r] = c < r ? v : c == r && r < T ? v + lift : 0.f;
         }
       }
       float dg = 0.f;
-      if (tid < T) dg = S.diag[S.perm[tid]] * sc;
+      if (tid < T) dg = S.diag[S.perm[tid]] * sc + lift;
       __syncthreads();
       if (tid < T) {
         S.diag[tid] = dg;
@@ -351,7 +366,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
     if (rank != 0) {
       for (int i = tid; i < T; i += nthr) S.perm[i] = __ldcg(&iscr[i]);
       if (pass == 0) {
-        const int pw = __ldcg(&gflag[8]);
+        const int pw = __ldcg(&gflag[15]);
         scale = exp2i(-pw);
         rootf = exp2i(-pw / 2);
       }
@@ -500,7 +515,8 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
     more = __syncthreads_or(more);
     if (more && tid == 0) atomicOr(&gflag[1 + pass], 1);
     eig_sync(nr);
-    const bool last = pass + 1 == kEigPasses || __ldcg(&gflag[1 + pass]) == 0;
+    unfinished = __ldcg(&gflag[1 + pass]) != 0;
+    const bool last = pass + 1 == kEigPasses || !unfinished;
     // ---- P = Vn - Vn C ----
     eig_product<RT, false>(T, ld, false, rank, nr, sm, smf, row(ES_VNT), none, row(ES_C), none,
                            [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
@@ -591,6 +607,8 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       ctrl->eig_phase_ns[2] += t3 - t2;
       ctrl->eig_phase_ns[3] += t4 - t3;
       ctrl->eig_rounds += sweeps * (jac_blocks(T) - 1);
+      ctrl->eig_further += pass;
+      ctrl->eig_unfinished += unfinished ? 1 : 0;
       set_cond(h, use_cond, 1u);
     }
   }

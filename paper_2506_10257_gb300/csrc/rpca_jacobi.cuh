@@ -91,12 +91,13 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 // t = s / c.  With dd = aqq - app and r = 1 / sqrt(dd^2 + 4 d^2), cos 2 theta =
 // |dd| r, so c^2 = (1 + |dd| r) / 2 and s = sign(dd) d r / c: two reciprocal
 // square roots in a row where the tangent's formula has three steps of that
-// length.  Returns the cosine.
+// length.  Two columns so short that dd^2 + 4 d^2 underflows are left alone too (the
+// formula would not be a rotation).  Returns the cosine.
 __device__ __forceinline__ float jac_rotation(float app, float aqq, float d, float& c, float& s, float& t) {
   const float cosv = fabsf(d) * (rsqrt_fast(fmaxf(app, 1e-37f)) * rsqrt_fast(fmaxf(aqq, 1e-37f)));
   const float dd = aqq - app, d2 = d + d;
-  const float r = rsqrt_fast(fmaxf(fmaf(dd, dd, d2 * d2), 1e-37f));
-  const bool act = cosv > kJacTol && cosv < 1.5f;  // (a zero column's cosine is zero; not a number is left alone)
+  const float q = fmaf(dd, dd, d2 * d2), r = rsqrt_fast(fmaxf(q, 1e-37f));
+  const bool act = cosv > kJacTol && cosv < 1.5f && q >= 1e-37f;  // (a zero column's cosine is zero; not a number is left alone)
   const float c2 = fmaf(0.5f * fabsf(dd), r, 0.5f);
   const float ic = rsqrt_fast(fmaxf(c2, 0.5f));
   c = act ? c2 * ic : 1.f;

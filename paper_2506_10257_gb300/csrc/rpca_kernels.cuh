@@ -1222,6 +1222,8 @@ static __global__ void begin_kernel(Bufs b, const float* X, float* L, float* S, 
     b.red->t_loop = 0ull;
     b.red->t_l1 = 0ull;
     c->eig_rounds = 0;
+    c->eig_further = 0;
+    c->eig_unfinished = 0;
     b.red->t_start = ~0ull;
     b.red->t_end = 0ull;
     b.red->err = 0;

@@ -28,7 +28,7 @@ MAX_T_NARROW = 32
 
 EXPORTED = ["rpca_params_default", "rpca_workspace_size", "rpca_plan_create", "rpca_solve", "rpca_solve_host",
             "rpca_plan_result", "rpca_plan_destroy", "rpca_status_str", "rpca_gram", "rpca_eig",
-            "rpca_gram_noalloc", "rpca_plan_timings", "rpca_batch_create", "rpca_batch_solve",
+            "rpca_gram_noalloc", "rpca_plan_timings", "rpca_plan_eig_rounds", "rpca_batch_create", "rpca_batch_solve",
             "rpca_batch_solve_host", "rpca_batch_tune", "rpca_batch_set_schedule", "rpca_batch_info", "rpca_batch_window_ctas", "rpca_batch_destroy", "rpca_batch_schedule",
             "rpca_server_create", "rpca_server_set_warm", "rpca_submit", "rpca_poll", "rpca_server_wait",
             "rpca_server_stats", "rpca_server_destroy", "rpca_prefilter_scratch_bytes", "rpca_prefilter",
@@ -109,6 +109,7 @@ def load(build_if_missing: bool = True):
     lib.rpca_prefilter.argtypes = [vp, i64, i32, ctypes.c_double, i32, vp, vp, vp, vp, vp, vp]
     lib.rpca_prefilter_highpass.argtypes = [vp, i64, i32, ctypes.c_double, i32, vp, vp, vp, vp, vp, vp]
     lib.rpca_plan_timings.argtypes = [vp, ctypes.POINTER(ctypes.c_double), i32]
+    lib.rpca_plan_eig_rounds.argtypes = [vp, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.rpca_batch_create.argtypes = [ctypes.POINTER(Params), i32, ctypes.POINTER(vp)]
     lib.rpca_batch_solve.argtypes = [vp, ctypes.POINTER(Window), vp, ctypes.POINTER(Result)]
     lib.rpca_batch_solve_host.argtypes = [vp, ctypes.POINTER(Window), vp, ctypes.POINTER(Result)]
@@ -257,6 +258,14 @@ class Plan:
         keys = ["eig_load_us", "eig_sweeps_us", "eig_rotprod_us", "eig_basis_us", "eig_rounds", "eigs_timed",
                 "pass_work_us", "pass_red1_us", "pass_red2_us"]
         return dict(zip(keys, list(buf)))
+
+    def eig_rounds(self) -> dict:
+        """Rounds the eigen-steps of the last solve took beyond their first, and steps that ran out of rounds."""
+        further, unfinished = ctypes.c_int32(), ctypes.c_int32()
+        st = self.lib.rpca_plan_eig_rounds(self.handle, ctypes.byref(further), ctypes.byref(unfinished))
+        if st != OK:
+            raise RpcaError(st, "rpca_plan_eig_rounds")
+        return {"further": further.value, "unfinished": unfinished.value}
 
     def result(self) -> dict:
         res = Result()
