@@ -12,7 +12,9 @@
 // "Error-free transformations of matrix multiplication", 2012; three FMAs a term
 // where a compensated sum takes eleven operations), and Vn, P and K are kept as
 // (hi, lo) pairs.  H and Gp, whose errors scale with the entries they belong to, are
-// plain FP32 in the form G U = G + G D, D = U - I.  With all of them in plain FP32
+// plain FP32 in the form G U = G + G D, D = U - I, but for the first step: its Gram is
+// not rotated, every entry holds the largest eigenvalue's share, and G, H and Gp are
+// (hi, lo) pairs there (Dot2, as in the narrow step).  With all of them in plain FP32
 // the error of L on 64 x 64 x 100 pixels and frames is five times as large.
 // The sigma > tau decision, g and mu are FP64.
 //
@@ -52,7 +54,7 @@ __host__ __device__ constexpr size_t eig_wide_smem(int T) {
 constexpr size_t kEigWMaxSmem = 216 * 1024;
 
 struct EigWideSh {
-  double d[kMaxTW];
+  double d[kMaxTW], mu_prev;
   float sig[kMaxTW], g1[kMaxTW], g1l[kMaxTW], diag[kMaxTW], piv[kMaxTW], nrm[kMaxTW];
   int perm[kMaxTW], keep[kMaxTW];
   unsigned smax[2], lift;
@@ -208,6 +210,52 @@ __device__ __forceinline__ void eig_product(int K, int ld, bool upper, int rank,
   __syncthreads();
 }
 
+// out = c + a^T b in two-float arithmetic for this rank's share of the T x T entries, four
+// rows a thread, of (hi, lo) pairs (a null low part: single floats), k increasing; upper:
+// only the entries with i <= j, mirrored.  Operands come from L2.  Run once a solve, and
+// not inlined, so that the body's own loops keep their place (132 columns, eight ranks: 0.2 ms
+// of a 30 ms solve).
+static __device__ __noinline__ void eig_product_dd(int T, int ld, bool upper, int rank, int nr, const float* a,
+                                                   const float* al, const float* b, const float* bl, const float* c,
+                                                   const float* cl, float* out, float* outl) {
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int g = rank * (int)blockDim.x + (int)threadIdx.x; g < (T + 3) / 4 * T; g += nr * (int)blockDim.x) {
+    const int i0 = g / T * 4, j = g % T;
+    if (upper && j < i0) continue;
+    float s[4], r[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      s[u] = __ldcg(&c[(i0 + u) * ld + j]);
+      r[u] = __ldcg(&cl[(i0 + u) * ld + j]);
+    }
+#pragma unroll 4
+    for (int k = 0; k < T; ++k) {
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(a + k * ld + i0));
+      const float4 xl = al ? __ldcg(reinterpret_cast<const float4*>(al + k * ld + i0)) : zero;
+      const float y = __ldcg(&b[k * ld + j]), yl = bl ? __ldcg(&bl[k * ld + j]) : 0.f;
+      const float xv[4] = {x.x, x.y, x.z, x.w}, xw[4] = {xl.x, xl.y, xl.z, xl.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        dot2(s[u], r[u], xv[u], y);
+        r[u] = fmaf(xv[u], yl, fmaf(xw[u], y, r[u]));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u;
+      if (i >= T || (upper && i > j)) continue;
+      float hi, lo;
+      fast_two_sum(s[u], r[u], hi, lo);
+      out[i * ld + j] = hi;
+      outl[i * ld + j] = lo;
+      if (upper) {
+        out[j * ld + i] = hi;
+        outl[j * ld + i] = lo;
+      }
+    }
+  }
+}
+
 // Sweeps for the window's column length.
 static __device__ __noinline__ int eig_wide_factor(float* W, int T, EigWideSh& S, float stop, float lim, int cap) {
   const int LD = jac_ld(T), nb = jac_blocks(T), r2 = jac_r2(T);
@@ -244,14 +292,24 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   const unsigned long long t0 = gtimer();
 
   // ---- the Gram, this rank's share of the sums over the CTAs of the pass ----
+  // (the first step's low parts lie where later matrices of the step go)
   float* G = M(ES_G);
+  enum { ES_GL = ES_B, ES_GSL = ES_C, ES_HL = ES_KT, ES_GPL = ES_KTL };
+  auto put_gram = [&](int e, float gh, float gl) {
+    float hi, lo;
+    fast_two_sum(gh, gl, hi, lo);
+    G[e / T * ld + e % T] = hi;
+    if (init) M(ES_GL)[e / T * ld + e % T] = lo;
+  };
   auto gram = [&](int i, int n) {
     const int e0 = (int)((int64_t)TT * rank / nr), e1 = (int)((int64_t)TT * (rank + 1) / nr);
     if (b.finalize) {
-      for (int e = e0 + i; e < e1; e += n) G[e / T * ld + e % T] = (float)__ldcg(&b.Gw[e]);
+      for (int e = e0 + i; e < e1; e += n) {
+        const double g = __ldcg(&b.Gw[e]);
+        put_gram(e, (float)g, (float)(g - (double)(float)g));
+      }
     } else if (__ldcg(&b.red->gram_last)) {
-      sum_rows<4, 8>(b.group_part, 0, __ldcg(&b.red->ngroups_last), TT,
-                  [&](int e, float gh, float gl) { G[e / T * ld + e % T] = gh + gl; }, i, n, e0, e1);
+      sum_rows<4, 8>(b.group_part, 0, __ldcg(&b.red->ngroups_last), TT, put_gram, i, n, e0, e1);
     }
   };
   bool go;
@@ -274,9 +332,8 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
   const float* vt = M(ES_VT);      // the basis, transposed
   float scale = 1.f, rootf = 1.f;
   int sweeps = 0, pass = 0;
-  bool unfinished = false;
   double tau = init ? 0.0 : __ldcg(&ctrl->inv_cur);
-  const double mu_prev = init ? __ldcg(&ctrl->mu_cur) : 0.0;  // (of the plan's previous solve)
+  if (init && tid == 0) S.mu_prev = __ldcg(&ctrl->mu_cur);  // (of the plan's previous solve; read by this thread)
   float tauf = 0.f;
   for (;; ++pass) {
     if (rank == 0) {
@@ -329,6 +386,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
           if (c < T && r < T) {
             v = __ldcg(&src[pc * ld + S.perm[r]]) * sc;
             M(ES_GS)[c * ld + r] = v;
+            if (init && pass == 0) M(ES_GSL)[c * ld + r] = __ldcg(&M(ES_GL)[pc * ld + S.perm[r]]) * sc;
           }
           sm[c * LD + r] = c < r ? v : c == r && r < T ? v + lift : 0.f;
         }
@@ -400,15 +458,18 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
             }
           }
         });
-    eig_product<RT, false>(T, ld, false, rank, nr, sm, smf, row(ES_GS), none, row(ES_D), none,
-                           [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
+    if (init && pass == 0)
+      eig_product_dd(T, ld, false, rank, nr, M(ES_GS), M(ES_GSL), M(ES_D), nullptr, M(ES_GS), M(ES_GSL), M(ES_H), M(ES_HL));
+    else
+      eig_product<RT, false>(T, ld, false, rank, nr, sm, smf, row(ES_GS), none, row(ES_D), none,
+                             [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
 #pragma unroll
-                             for (int i = 0; i < RT; ++i) {
-                               const float4 g = __ldcg(reinterpret_cast<const float4*>(M(ES_GS) + (i0 + i) * ld + j0));
-                               *reinterpret_cast<float4*>(M(ES_H) + (i0 + i) * ld + j0) =
-                                   make_float4(g.x + acc[i][0], g.y + acc[i][1], g.z + acc[i][2], g.w + acc[i][3]);
-                             }
-                           });
+                               for (int i = 0; i < RT; ++i) {
+                                 const float4 g = __ldcg(reinterpret_cast<const float4*>(M(ES_GS) + (i0 + i) * ld + j0));
+                                 *reinterpret_cast<float4*>(M(ES_H) + (i0 + i) * ld + j0) =
+                                     make_float4(g.x + acc[i][0], g.y + acc[i][1], g.z + acc[i][2], g.w + acc[i][3]);
+                               }
+                             });
     eig_sync(nr);
     // ---- Omega = Vn^T Vn - I, Gp = U^T H = H + D^T H (upper triangles, mirrored) ----
     eig_product<RT, true>(T, ld, true, rank, nr, sm, smf, row(ES_VN), row(ES_VNL), row(ES_VN), row(ES_VNL),
@@ -424,23 +485,26 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
                                 M(ES_OM)[q * ld + p] = v;
                               }
                           });
-    eig_product<RT, false>(T, ld, true, rank, nr, sm, smf, row(ES_D), none, row(ES_H), none,
-                           [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
+    if (init && pass == 0)
+      eig_product_dd(T, ld, true, rank, nr, M(ES_D), nullptr, M(ES_H), M(ES_HL), M(ES_H), M(ES_HL), M(ES_GP), M(ES_GPL));
+    else
+      eig_product<RT, false>(T, ld, true, rank, nr, sm, smf, row(ES_D), none, row(ES_H), none,
+                             [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
 #pragma unroll
-                             for (int i = 0; i < RT; ++i)
+                               for (int i = 0; i < RT; ++i)
 #pragma unroll
-                               for (int j = 0; j < 4; ++j) {
-                                 const int p = i0 + i, q = j0 + j;
-                                 if (p > q) continue;
-                                 const float v = __ldcg(&M(ES_H)[p * ld + q]) + acc[i][j];
-                                 M(ES_GP)[p * ld + q] = v;
-                                 M(ES_GP)[q * ld + p] = v;
-                               }
-                           });
+                                 for (int j = 0; j < 4; ++j) {
+                                   const int p = i0 + i, q = j0 + j;
+                                   if (p > q) continue;
+                                   const float v = __ldcg(&M(ES_H)[p * ld + q]) + acc[i][j];
+                                   M(ES_GP)[p * ld + q] = v;
+                                   M(ES_GP)[q * ld + p] = v;
+                                 }
+                             });
     eig_sync(nr);
     // ---- FP64 decisions (every rank makes the same ones) ----
     for (int i = tid; i < T; i += nthr) {
-      const double gp = (double)__ldcg(&M(ES_GP)[i * ld + i]);
+      const double gp = (double)__ldcg(&M(ES_GP)[i * ld + i]) + (init && pass == 0 ? (double)__ldcg(&M(ES_GPL)[i * ld + i]) : 0.0);
       S.d[i] = gp - gp * (double)__ldcg(&M(ES_OM)[i * ld + i]);
     }
     __syncthreads();
@@ -448,7 +512,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       if (rank == 0 && tid == 0) {
         double lmax = 0.0;
         for (int a = 0; a < T; ++a) lmax = fmax(lmax, S.d[a]);
-        init_mu(b, lmax / (double)scale, mu_prev);
+        init_mu(b, lmax / (double)scale, S.mu_prev);
       }
       eig_sync(nr);
       tau = __ldcg(&ctrl->inv_cur);
@@ -471,6 +535,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
     }
     __syncthreads();
     // ---- C, -F o E, E, and whether E (beyond its FP32 rounding) and Omega are small enough ----
+    const float noise = init ? 0.f : kEigNoise;
     int more = 0;
     for (int p = rank + nr * warp; p < T; p += nr * nwarps) {
       float most = 0.f;
@@ -487,11 +552,11 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
         const float sq = S.sig[q], dq = (float)S.d[q];
         const bool pbig = S.d[p] > S.d[q] || (S.d[p] == S.d[q] && p < q);
         const float hi = fmaxf(sp, sq), lo = fminf(sp, sq), dm = pbig ? dp : dq;
-        const float ev = fmaf(-dm, om, __ldcg(&M(ES_GP)[p * ld + q]));
+        const float ev = fmaf(-dm, om, __ldcg(&M(ES_GP)[p * ld + q])) + (init && pass == 0 ? __ldcg(&M(ES_GPL)[p * ld + q]) : 0.f);
         M(ES_C)[p * ld + q] = pbig ? om : 0.f;
         M(ES_B)[p * ld + q] = -g_divided_difference(hi, lo, tauf) * ev;
         M(ES_E)[p * ld + q] = ev;
-        const float e = fmaxf(fabsf(ev) - kEigNoise * dm, 0.f);
+        const float e = fmaxf(fabsf(ev) - noise * dm, 0.f);
         const int kept = kp + S.keep[q];
         if (kept && eig_pair_off(e, fabsf(om), hi, lo, kept)) more = 1;
         if (kept != 1) most += eig_pair_most(e, fabsf(om), hi);
@@ -506,7 +571,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
         for (int q = lane; q < T; q += 32) {
           if (q == p || S.keep[q] != kp) continue;
           const float sq = S.sig[q], dm = fmaxf(dp, (float)S.d[q]);
-          const float e = fmaxf(fabsf(M(ES_E)[p * ld + q]) - kEigNoise * dm, 0.f);  // (this lane's own store)
+          const float e = fmaxf(fabsf(M(ES_E)[p * ld + q]) - noise * dm, 0.f);  // (this lane's own store)
           shift += eig_pair_shift(e, fabsf(__ldcg(&M(ES_OM)[p * ld + q])), fmaxf(sp, sq), fminf(sp, sq));
         }
         if (row_off(shift)) more = 1;
@@ -515,8 +580,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
     more = __syncthreads_or(more);
     if (more && tid == 0) atomicOr(&gflag[1 + pass], 1);
     eig_sync(nr);
-    unfinished = __ldcg(&gflag[1 + pass]) != 0;
-    const bool last = pass + 1 == kEigPasses || !unfinished;
+    const bool last = pass + 1 == kEigPasses || __ldcg(&gflag[1 + pass]) == 0;
     // ---- P = Vn - Vn C ----
     eig_product<RT, false>(T, ld, false, rank, nr, sm, smf, row(ES_VNT), none, row(ES_C), none,
                            [&](int i0, int j0, float (&acc)[RT][4], float (&)[RT][4]) {
@@ -608,7 +672,7 @@ static __device__ void eig_wide_body(Bufs b, int flags, cudaGraphConditionalHand
       ctrl->eig_phase_ns[3] += t4 - t3;
       ctrl->eig_rounds += sweeps * (jac_blocks(T) - 1);
       ctrl->eig_further += pass;
-      ctrl->eig_unfinished += unfinished ? 1 : 0;
+      ctrl->eig_unfinished += __ldcg(&gflag[1 + pass]);
       set_cond(h, use_cond, 1u);
     }
   }

@@ -68,5 +68,19 @@ def test_nearly_low_rank_windows_keep_fp32_rounding(rp, T, noise):
     assert eL <= bar and eS <= bar, (eL / bar, eS / bar)
 
 
+@pytest.mark.parametrize("T", [40, 50, 100, 132])
+def test_first_wide_step_resolves_what_its_gram_holds(rp, T):
+    # singular values that span 1e4 in the first, unrotated Gram, all of them above tau: G, H and Gp need more than FP32
+    # there (bar: the reduced precisions' 1e-4 of ||X||; in FP32 3e-4)
+    F = low_noise(T, 2048, 1e-3)
+    mu = 1e5 * 1.25 / np.linalg.norm(F.astype(np.float64), 2)
+    plan = rp.Plan(2048, T, mu_init=mu)
+    L, S, res = plan.solve(torch.from_numpy(F).cuda())
+    plan.close()
+    ref = O.rpca_frames(F, mu_init=mu, max_iter=res["iters"], tol=1e-30)
+    eL = np.linalg.norm(L.cpu().numpy() - ref.L)
+    assert eL <= 1e-4 * np.linalg.norm(F), (eL / np.linalg.norm(F), res["iters"])
+
+
 def test_eig_rounds_checks_its_arguments(rp):
     assert rp.load().rpca_plan_eig_rounds(None, None, None) == rp.ERR_ARG
