@@ -197,8 +197,8 @@ static __device__ __noinline__ bool eig64_body(Bufs b, int flags, cudaGraphCondi
       for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
       if (lane < T) S.U[lane * LD + c] = n > 0.f ? x * rsqrtf(n) : (lane == c ? 1.f : 0.f);
     }
-    if (tid < 2) S.smax[tid] = 0u;
     __syncthreads();
+    if (tid < 2) S.smax[tid] = 0u;  // (every warp has left the sweeps)
     if (tid == 0) S.lift = 0u;
     t2 = gtimer();
     // ---- Vn = V U, H = G U ----

@@ -132,7 +132,8 @@ __device__ __forceinline__ void jac_within(uint64_t (&a)[R2], float& na, int x, 
 // (what such a sweep leaves is quadratically smaller), and none of two shorter
 // columns above stop / kJacFar (they must stay a basis), or for max_sweeps sweeps.
 // nrm: 4 nb floats; smax: two words, zero on entry.  All threads of the CTA call
-// it (after a barrier) and get the number of sweeps; it ends with a barrier.
+// it (after a barrier) and get the number of sweeps; smax is read after its last
+// barrier, so the caller resets it after one of its own.
 template <int R2>
 static __device__ __noinline__ int jac_sweeps(float* W, int LD, int nb, float* nrm, unsigned* smax, float stop, float t2,
                                               int max_sweeps) {
