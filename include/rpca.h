@@ -55,8 +55,11 @@ typedef enum {
 typedef enum { RPCA_R32 = 0, RPCA_C64 = 1 } rpca_dtype;
 
 /* Arithmetic of the two dense contractions per iteration (Z*Wbar and the
- * rotated Gram).  The eigensolve, the sigma-vs-tau decision, mu and the
- * convergence test are FP64 in every mode. */
+ * rotated Gram).  In every mode the sigma-vs-tau decision, mu and the
+ * convergence test are FP64, and the eigensolve proposes its vectors in FP32
+ * and forms what it returns by products that carry more: two-float (hi, lo)
+ * sums up to 32 real columns; beyond, operands split so that the leading sums
+ * are exact, FP32 where an entry's error scales with the entry. */
 typedef enum {
   RPCA_PREC_FP32 = 0,       /* FP32 CUDA-core FMA */
   RPCA_PREC_TF32X3 = 1,     /* tensor cores, TF32 hi/lo split, 3 products, FP32 accumulate */
@@ -113,7 +116,8 @@ typedef struct {
 } rpca_params;
 
 /* Largest frame count.  Windows of T <= 32 frames run one pixel row per
- * thread; T in 33..224 run the shared-memory tiled path (FP32 only). */
+ * thread; T in 33..224 run the shared-memory tiled path (the tensor-core
+ * precisions up to 128 real columns). */
 #define RPCA_MAX_T 224
 #define RPCA_MAX_T_NARROW 32
 

@@ -102,7 +102,7 @@ struct Layout {
       total;
   int grid, ngroups, group;
   int ws_grid;     // CTAs of the passes with 128-pixel tiles (TMA-fed FP32, tiled tensor-core): one per SM
-  int wide_grid;   // CTAs of the wide pass (T > kMaxT; one per SM, 32-pixel tiles)
+  int wide_grid;   // CTAs of the tiled pass (one per SM, 64- or 128-pixel tiles)
 };
 
 int device_sms() {
@@ -202,7 +202,7 @@ rpca_status validate(const rpca_params* p) {
 struct rpca_plan_s {
   rpca_params p;
   KernelSet ks;
-  bool wide;          // T > kMaxT: shared-memory tiled passes, 1024-thread eigen-step
+  bool wide;          // T > kMaxT or complex: tiled passes, and beyond kMaxT columns the eigen-step of a cluster
   WideKernels wk;
   Layout lay;
   Bufs bufs;

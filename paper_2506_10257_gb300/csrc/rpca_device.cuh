@@ -148,7 +148,7 @@ struct Bufs {
   int wide;            // tiled path: the reduced Gram goes to Gw (T x T), else to red->G (kMaxT stride)
   int finalize;        // 1: the pass itself sums the group partials into red->G, e2, l1;
                        // 0: the next eigen-step does (saves a serial reduction level)
-  // T > kMaxT ("wide" windows): the reduced Gram, Wbar and V live in these
+  // Windows of the tiled path (b.wide): the reduced Gram, Wbar and V live in these
   // T x T row-major arrays of the workspace instead of red->G and EigState.
   double* Gw;          // summed partial Grams as FP64 (also scratch of the eigen-step)
   float* Ww;

@@ -474,11 +474,6 @@ __device__ __forceinline__ void cp_async4(float* sdst, const float* gsrc) {
                "l"(gsrc)
                : "memory");
 }
-__device__ __forceinline__ void cp_async16(float* sdst, const float* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(sdst)),
-               "l"(gsrc)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
