@@ -133,7 +133,7 @@ struct NarrowBody {
   static __device__ bool pass(Bufs b, bool init, int lc, int nc, unsigned char* dsm) {
     return init ? pass_body<TB, PM_INIT>(b, lc, nc, dsm) : pass_body<TB, PM_FUSED>(b, lc, nc, dsm);
   }
-  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int) { eig64_body(b, flags, 0, 0, dsm); }
+  static __device__ void eig(Bufs b, int flags, unsigned char* dsm, int) { eig64_body<false>(b, flags, 0, 0, dsm); }
 };
 
 // The window's state reset before its solve (the lane's CTA 0, thread 0).

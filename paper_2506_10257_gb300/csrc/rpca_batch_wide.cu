@@ -53,7 +53,7 @@ struct WideDisp {
     // (up to 32 columns: the narrow step, as in plans; a batch of four 8-frame complex
     // 100 x 100 windows takes 2.1 ms, 4.2 with the wide one)
     if (wd.b.T <= kMaxT)
-      eig64_body(wd.b, flags, 0, 0, dsm);
+      eig64_body<false>(wd.b, flags, 0, 0, dsm);
     else
       wide_eig_call(wd.b, flags, reinterpret_cast<float*>(dsm), eig_floats);
   }

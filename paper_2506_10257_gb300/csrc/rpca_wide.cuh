@@ -673,7 +673,7 @@ __device__ __forceinline__ void wtc_images(const Bufs& b, const float* v, int sn
 static __global__ void __launch_bounds__(kEigThreads) eig_small_kernel(Bufs b, int flags, cudaGraphConditionalHandle h,
                                                                        int use_cond, int) {
   extern __shared__ __align__(16) unsigned char eigs_smem[];
-  if (eig64_body(b, flags, h, use_cond, eigs_smem) && b.wtc) {
+  if (eig64_body<true>(b, flags, h, use_cond, eigs_smem) && b.wtc) {
     __syncthreads();  // Ww and Vw written
     wtc_images(b, b.Vw, 1, b.T, 0, 1);
   }
