@@ -25,8 +25,9 @@
 // and the sweeps stop once what is neglected is about the result's FP32 rounding,
 // the kink of f at tau included (rpca_eig_rule.cuh).  A step that finds more left
 // runs another round of sweeps on diag(d) + E.  sigma, the sigma > tau decision, g and mu are FP64.  Measured on
-// the windows above: 25 us (load 3, factor and sweeps 13, products and decisions 10)
-// and 44 us, at the same errors of L and S against 64 bits (1.0e-7 and 2.3e-7).
+// the windows above: 26 us (load 3, factor and sweeps 13, products and decisions 10)
+// and 38 to 40 us, at 0.84 to 0.95 of the errors of L and S against 64 bits (means of
+// 12 seeds: 1.0e-7 and 2.2e-7).
 #pragma once
 
 constexpr int kEigThreads = 256;   // threads of the eigen-step CTA

@@ -24,9 +24,9 @@
 // rows, with every T x T operand in the workspace (L2) and a cluster barrier
 // between products.  Bound by the factor and the sweeps on rank 0's SM, which wait
 // at its barriers.  Measured with 8 ranks, against cyclic Jacobi on the Gram itself:
-// 50 frames 295 -> 118 us (factor and sweeps 47, products 47), 100 frames
-// 1106 -> 273 us (170, 63), 132 frames 2310 -> 491 us (353, 92).  One CTA, beside
-// the other lanes of a batch, takes 220 us at 63 frames and 405 us at 93.
+// 50 frames 294 -> 124 us (factor and sweeps 50, products 50), 100 frames
+// 1106 -> 273 us (168, 66), 132 frames 2313 -> 512 to 550 us (366 to 410, 96).  One CTA,
+// beside the other lanes of a batch, takes 238 us at 63 frames and 437 us at 93.
 #pragma once
 
 // Matrices of the step's scratch, each eig_ld(T)^2 floats.
